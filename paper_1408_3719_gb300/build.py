@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libaleweno.so")
-SOURCES = ["aw_host.cu", "aw_kernels.cu", "aw_noalloc.cu", "aw_adjoint.cu"]
+SOURCES = ["aw_host.cu", "aw_kernels.cu", "aw_plain.cu", "aw_noalloc.cu", "aw_adjoint.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off"]
 

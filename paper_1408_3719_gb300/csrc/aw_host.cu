@@ -29,7 +29,7 @@ struct aw_ctx {
   std::vector<void*> allocs;
   Counters* hcnt = nullptr;  // pinned mirror of the device counters
   bool prof = false;         // per-kernel CUDA-event timing of sweeps
-  cudaGraphExec_t prof_graph = nullptr;  // the sweep with an event before and after every kernel
+  cudaGraphExec_t prof_graph[2] = {};  // the sweep with an event before and after every kernel
   cudaEvent_t prof_ev[kNumKernels + 1] = {};
   // side stream of the sweep graph: the node solver runs beside the edge
   // marking (they read the moved-node list and write disjoint arrays)
@@ -41,7 +41,7 @@ struct aw_ctx {
   std::vector<double> xy0;
   double* d_corner0 = nullptr;  // element corners at t = 0
   std::vector<double> etick_h, ntick_h;  // seconds per tick of each element / node
-  cudaGraphExec_t graph_exec = nullptr;  // one captured sweep
+  cudaGraphExec_t graph_exec[2] = {};  // one captured sweep: the fast and the plain kernels (Dev::plain)
   Tiles tiles;                           // tile shapes of the sweep kernels
   std::vector<int> tri_h;                // host copies for aw_load_state_xy
   std::vector<double> cshift_h;
@@ -319,6 +319,36 @@ int build_tab(aw_ctx* c) {
     }
   }
   return AW_OK;
+}
+
+PredTab pred_tab(const Tab& T) {
+  PredTab P{};
+  const int M = T.M;
+  for (int t = 0; t < T.Nt; ++t)
+    for (int u = 0; u < T.Nt; ++u) {
+      P.Dtau[t][u] = T.Dtau[t][u];
+      P.Vt[t][u] = T.VtInv[t][u];
+      if (t + 1 < T.Nt) {
+        P.B[t][u] = T.B[t][u];
+        P.B[t][kMaxNt] += T.B[t][u];
+      }
+    }
+  for (int s = 0; s < T.Mc; ++s) {
+    P.wavg[s] = T.wavg[s];
+    for (int c = 0; c < 2; ++c) P.lat[s][c] = T.lat[s][c];
+    for (int r = 0; r < T.Mc; ++r) {
+      P.dx[s][r] = (float)std::rint(2.0 * T.Dxi[s][r]);
+      P.de[s][r] = (float)std::rint(2.0 * T.Deta[s][r]);
+    }
+  }
+  // node c of edge e on the lattice: (i, j) = (c, 0), (M - c, c), (0, M - c)
+  for (int e = 0; e < 3; ++e)
+    for (int c = 0; c < T.Nt; ++c) {
+      const int j = e == 0 ? 0 : (e == 1 ? c : M - c), i = e == 0 ? c : (e == 1 ? M - c : 0);
+      P.en[e][c] = j * (M + 1) - j * (j - 1) / 2 + i;
+      for (int g = 0; g < T.Nt; ++g) P.W[e * T.Nt + g][c] = T.Tr[e][g][P.en[e][c]];
+    }
+  return P;
 }
 
 // ---------------------------------------------------------------------------
@@ -630,13 +660,10 @@ int dupload(aw_ctx* c, const T** out, const std::vector<T>& v) {
 // the captured sweeps become invalid when the tiles, the schedule mode or the
 // mesh change
 void drop_graphs(aw_ctx* c) {
-  if (c->graph_exec) {
-    cudaGraphExecDestroy(c->graph_exec);
-    c->graph_exec = nullptr;
-  }
-  if (c->prof_graph) {
-    cudaGraphExecDestroy(c->prof_graph);
-    c->prof_graph = nullptr;
+  for (int k = 0; k < 2; ++k) {
+    if (c->graph_exec[k]) cudaGraphExecDestroy(c->graph_exec[k]);
+    if (c->prof_graph[k]) cudaGraphExecDestroy(c->prof_graph[k]);
+    c->graph_exec[k] = c->prof_graph[k] = nullptr;
   }
 }
 
@@ -918,6 +945,8 @@ static int load_common(aw_ctx* c, int64_t n_nodes, const double* xy, int64_t n_t
   for (int i = 0; i < m.ne; ++i)
     for (int k = 0; k < 3; ++k) c->ntick_h[m.tri[3 * i + k]] = c->etick_h[i];
   if ((rc = dupload(c, &d.etick, c->etick_h))) return rc;
+  const std::vector<PredTab> ptab(1, pred_tab(T));
+  if ((rc = dupload(c, &d.ptab, ptab))) return rc;
   const size_t ne = m.ne, nn = m.nn, ned = m.ned;
   if ((rc = dalloc(c, &d.Q, 4 * ne)) || (rc = dalloc(c, &d.QM, 4 * ne)) || (rc = dalloc(c, &d.HM, 4 * ne)) ||
       (rc = dalloc(c, &d.t, ne)) || (rc = dalloc(c, &d.dt, ne)) || (rc = dalloc(c, &d.X, 6 * ne)) ||
@@ -1044,6 +1073,7 @@ static int load_state_impl(aw_ctx* c, const double* Q, const double* xy) {
     CK(cudaStreamSynchronize(c->stream));
   }
 
+  d.plain = xy ? 1 : 0;
   launch_initial(c->tab, d, c->nsm, c->stream, c->tiles);
   CK(cudaGetLastError());
   int rc = sync_counters(c);
@@ -1074,7 +1104,9 @@ static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
   // With profiling it is a second graph with an event record between the
   // kernels: each profiled sweep waits for its last event and adds the
   // kernel times (the kernels run as in the plain graph).
-  if (!c->prof && !c->graph_exec) {
+  cudaGraphExec_t& graph = c->graph_exec[c->d.plain];
+  cudaGraphExec_t& prof_graph = c->prof_graph[c->d.plain];
+  if (!c->prof && !graph) {
     if (!c->side) {
       CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
       CK(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
@@ -1084,22 +1116,22 @@ static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     launch_sweep(c->tab, c->d, c->nsm, c->stream, nullptr, c->tiles, c->side, c->fork_ev, c->join_ev);
     CK(cudaStreamEndCapture(c->stream, &g));
-    CK(cudaGraphInstantiate(&c->graph_exec, g, 0));
+    CK(cudaGraphInstantiate(&graph, g, 0));
     cudaGraphDestroy(g);
   }
-  if (c->prof && !c->prof_graph) {
+  if (c->prof && !prof_graph) {
     for (cudaEvent_t& e : c->prof_ev)
       if (!e) CK(cudaEventCreate(&e));
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     launch_sweep(c->tab, c->d, c->nsm, c->stream, c->prof_ev, c->tiles);
     CK(cudaStreamEndCapture(c->stream, &g));
-    CK(cudaGraphInstantiate(&c->prof_graph, g, 0));
+    CK(cudaGraphInstantiate(&prof_graph, g, 0));
     cudaGraphDestroy(g);
   }
   for (int64_t k = 0; k < n; ++k) {
     if (c->prof) {
-      CK(cudaGraphLaunch(c->prof_graph, c->stream));
+      CK(cudaGraphLaunch(prof_graph, c->stream));
       CK(cudaEventSynchronize(c->prof_ev[kNumKernels]));
       for (int q = 0; q < kNumKernels; ++q) {
         float ms = 0.0f;
@@ -1108,7 +1140,7 @@ static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
       }
       c->prof_sweeps += 1;
     } else {
-      CK(cudaGraphLaunch(c->graph_exec, c->stream));
+      CK(cudaGraphLaunch(graph, c->stream));
     }
   }
   CK(cudaGetLastError());
@@ -1295,6 +1327,7 @@ int aw_set_elem_arrays(aw_ctx* c, const double* Q, const double* QM, const doubl
   if (rc0) return rc0;
   if ((rc0 = count_unfinished(c, nullptr))) return rc0;
 
+  c->d.plain = 0;
   launch_products(c->tab, c->d, c->nsm, c->stream);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->stream));
@@ -1439,6 +1472,7 @@ int aw_adjoint_forward(aw_ctx* c, int64_t n_sweeps, int64_t ckpt_every) {
   for (auto& s : c->slots)
     if ((rc = snap_alloc(c, &s))) return rc;
   c->last_seg_kept = false;
+  c->d.plain = 1;
   if ((rc = snap_copy(c, c->ckpt[0], true))) return rc;
   // the last segment is the first one the reverse pass needs: keep its
   // sweep-start states now instead of recomputing them

@@ -43,6 +43,21 @@ struct Tab {
   double glx[kMaxNt], glw[kMaxNt];
 };
 
+// The predictor's reference tables in device memory, laid out as its blocks
+// hold them: a block copies them with one 16-byte load per thread, where
+// indexing the parameter bank by thread costs one replay per distinct address
+// (8,000 of the 34,000 cycles of a block with one element at order M = 3).
+struct alignas(16) PredTab {
+  double B[kMaxNt - 1][kMaxNt + 1];     // column Nt: the row sum
+  double Dtau[kMaxNt][kMaxNt], Vt[kMaxNt][kMaxNt];
+  double W[3 * kMaxNt][kMaxNt];         // an edge's Gauss-point values from its M + 1 nodes
+  double wavg[kMaxMc], lat[kMaxMc][2];
+  double pad_;
+  float dx[kMaxMc][kMaxMc], de[kMaxMc][kMaxMc];  // twice the nodal derivative weights: integers
+  int en[3][kMaxNt];                    // lattice index of an edge's nodes, from its first vertex
+};
+static_assert(sizeof(PredTab) % 16 == 0, "PredTab is copied in 16-byte words");
+
 // Device-resident context data (pointers into one context's allocations).
 struct Dev {
   int ne, nn, ned, periodic;
@@ -72,6 +87,8 @@ struct Dev {
   const unsigned char* sten;  // [ne][7][n_e] local member index (0 = i itself)
   const signed char* sten_ok; // [ne*7]
   const double* etick;     // [ne] seconds per tick of the element's instance
+  const PredTab* ptab;
+  int plain;               // heavy kernels in plain FP64 (aw_plain.cu): a differentiated run
   // element state
   double* Q;     // [ne*4]
   double* QM;    // [ne*4]
@@ -173,6 +190,8 @@ void launch_sync_cut(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long
 // a new sync time above the current one Told: the elements stopped at Told get
 // their phase B (reconstruction, step, predictor)
 void launch_sync_resume(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long long Told, const Tiles& tl);
+// the same kernels' plain FP64 forms (aw_plain.cu)
+void launch_plain_predict(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 double measure_fp64_peak();
 // k_ready, k_nodes, k_edges of one sweep: ready/moved/active/touched lists
 // and the new node positions, without changing the state

@@ -927,6 +927,7 @@ static int load_common(aw_ctx* c, int64_t n_nodes, const double* xy, int64_t n_t
   Dev& d = c->d;
   d = Dev{};
   d.ne = m.ne; d.nn = m.nn; d.ned = m.ned; d.periodic = m.periodic;
+  for (int i = 0; i < m.ne; ++i) d.max_u = std::max(d.max_u, m.u_ptr[i + 1] - m.u_ptr[i]);
   d.period[0] = m.period[0]; d.period[1] = m.period[1];
   const Tab& T = c->tab;
   if ((rc = dupload(c, &d.tri, m.tri)) || (rc = dupload(c, &d.cshift, m.cshift)) || (rc = dupload(c, &d.elem_edge, m.elem_edge)) ||
@@ -946,7 +947,11 @@ static int load_common(aw_ctx* c, int64_t n_nodes, const double* xy, int64_t n_t
     for (int k = 0; k < 3; ++k) c->ntick_h[m.tri[3 * i + k]] = c->etick_h[i];
   if ((rc = dupload(c, &d.etick, c->etick_h))) return rc;
   const std::vector<PredTab> ptab(1, pred_tab(T));
-  if ((rc = dupload(c, &d.ptab, ptab))) return rc;
+  std::vector<ReconTab> rtab(1, ReconTab{});
+  std::memcpy(rtab[0].Bnod, T.Bnod, sizeof T.Bnod);
+  std::memcpy(rtab[0].SigU, T.SigU, sizeof T.SigU);
+  std::memcpy(rtab[0].mbar, T.mbar, sizeof T.mbar);
+  if ((rc = dupload(c, &d.ptab, ptab)) || (rc = dupload(c, &d.rtab, rtab))) return rc;
   const size_t ne = m.ne, nn = m.nn, ned = m.ned;
   if ((rc = dalloc(c, &d.Q, 4 * ne)) || (rc = dalloc(c, &d.QM, 4 * ne)) || (rc = dalloc(c, &d.HM, 4 * ne)) ||
       (rc = dalloc(c, &d.t, ne)) || (rc = dalloc(c, &d.dt, ne)) || (rc = dalloc(c, &d.X, 6 * ne)) ||

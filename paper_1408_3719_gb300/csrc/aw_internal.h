@@ -58,9 +58,16 @@ struct alignas(16) PredTab {
 };
 static_assert(sizeof(PredTab) % 16 == 0, "PredTab is copied in 16-byte words");
 
+// the reconstruction's tables, likewise
+struct alignas(16) ReconTab {
+  double Bnod[kMaxMc][kMaxNU], SigU[kMaxNU][kMaxNU], mbar[kMaxNU];
+};
+static_assert(sizeof(ReconTab) % 16 == 0, "ReconTab is copied in 16-byte words");
+
 // Device-resident context data (pointers into one context's allocations).
 struct Dev {
   int ne, nn, ned, periodic;
+  int max_u;               // largest number of distinct stencil members of an element
   double period[2];
   // mesh
   const int* tri;          // [ne*3]
@@ -88,6 +95,7 @@ struct Dev {
   const signed char* sten_ok; // [ne*7]
   const double* etick;     // [ne] seconds per tick of the element's instance
   const PredTab* ptab;
+  const ReconTab* rtab;
   int plain;               // heavy kernels in plain FP64 (aw_plain.cu): a differentiated run
   // element state
   double* Q;     // [ne*4]
@@ -191,6 +199,7 @@ void launch_sync_cut(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long
 // their phase B (reconstruction, step, predictor)
 void launch_sync_resume(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long long Told, const Tiles& tl);
 // the same kernels' plain FP64 forms (aw_plain.cu)
+void launch_plain_recon(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 void launch_plain_predict(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 double measure_fp64_peak();
 // k_ready, k_nodes, k_edges of one sweep: ready/moved/active/touched lists

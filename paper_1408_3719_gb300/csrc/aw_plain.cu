@@ -10,12 +10,60 @@
 // the predictor's roundings change, while the run's own state moves by 1e-15;
 // with these kernels it reproduces.
 #include <algorithm>
+#include <cfloat>
+#include <climits>
 
 #include "aw_internal.h"
 
 namespace aw {
 
 namespace {
+
+__device__ __forceinline__ double area6(const double* X) {
+  return 0.5 * ((X[2] - X[0]) * (X[5] - X[1]) - (X[3] - X[1]) * (X[4] - X[0]));
+}
+
+__device__ __forceinline__ void set_error(Counters* cnt, int code, int elem) {
+  if (atomicCAS(&cnt->err_code, 0, code) == 0) cnt->err_elem = elem;
+}
+
+__device__ __forceinline__ double pressure(const Tab& T, const double* q) {
+  return (T.gamma - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
+}
+
+// ---------------------------------------------------------------------------
+// virtual data of element j at time ti (ticks): eqs. virtGeom, virtCellaverage
+template <int M>
+__device__ __forceinline__ void virtual_data(const Tab& T, const Dev& d, int j, long long ti, double* Xv, double* Qv) {
+  constexpr int Nt = M + 1;
+  const long long tj = d.t[j], dtj = d.dt[j];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Xv[k] = d.X[6 * j + k];
+  if (tj == ti || dtj == 0) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Qv[v] = d.Q[4 * j + v];
+    return;
+  }
+  const double tau = (double)(ti - tj) * (1.0 / (double)dtj);  // a reciprocal costs half a divide
+  const double dts = (double)dtj * d.etick[j];
+  const double* vd = d.vdisp + (size_t)j * 6 * Nt;
+#pragma unroll
+  for (int kc = 0; kc < 6; ++kc) {
+    const double* c0 = vd + kc * Nt;
+    double acc = c0[Nt - 1];
+#pragma unroll
+    for (int p = Nt - 2; p >= 0; --p) acc = acc * tau + c0[p];
+    Xv[kc] += dts * (acc * tau);
+  }
+  const double* av = d.avgc + (size_t)j * Nt * 4;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    double acc = av[(Nt - 1) * 4 + v];
+#pragma unroll
+    for (int p = Nt - 2; p >= 0; --p) acc = acc * tau + av[p * 4 + v];
+    Qv[v] = acc;
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Cooperative predictor: one thread per (element, space-time node), G
@@ -317,6 +365,535 @@ __global__ void __launch_bounds__(TH, TH >= 256 ? 2 : 3) k_predict_coop(Tab T, D
   }
 }
 
+// ---------------------------------------------------------------------------
+// Cooperative reconstruction: G ready elements per 256-thread block; each
+// phase flattens its work items over the block (stencil members, normal-
+// equation entries, stencils, characteristic fields, output nodes).
+// ---------------------------------------------------------------------------
+template <int M>
+constexpr int recon_g_default() { return M == 1 ? 16 : (M == 2 ? 8 : 4); }
+
+template <int M, int GG = recon_g_default<M>()>
+struct ReconShape {
+  static constexpr int Mc = (M + 1) * (M + 2) / 2, NU = Mc - 1, NE = 2 * Mc;
+  static constexpr int MaxU = kNSten * (NE - 1);
+  static constexpr int G = GG;
+  // the default shape on 256 threads; half the elements on 128 threads (the
+  // same threads per element, twice the blocks and barrier domains per SM)
+  static constexpr int kThreads = GG < recon_g_default<M>() ? 128 : 256;
+  static constexpr int NL = NU * (NU + 1) / 2;      // lower triangle of the normal matrix
+  static constexpr int NN = NL + 4 * NU;           // + right-hand sides
+  static constexpr int RW = NU + 4;                 // row: basis averages, then Q~ - Q_i
+  static constexpr size_t oRow = 0;
+  static constexpr size_t oNrm = oRow + (size_t)G * (MaxU + 1) * RW;
+  static constexpr size_t oC = oNrm + (size_t)G * kNSten * NN;
+  static constexpr size_t oCh = oC + (size_t)G * kNSten * NU * 4;
+  static constexpr size_t oSig = oCh + (size_t)G * kNSten * NU * 4;
+  static constexpr size_t oWc = oSig + (size_t)G * kNSten * 4;
+  static constexpr size_t oCv = oWc + (size_t)G * NU * 4;
+  static constexpr size_t oRL = oCv + (size_t)G * NU * 4;
+  static constexpr size_t oEl = oRL + (size_t)G * 32;   // X(6), Q(4), Jinv(4)
+  static constexpr size_t oDt = oEl + (size_t)G * 16;
+  static constexpr size_t oBn = oDt + (size_t)G * 4;    // Bnod [Mc][NU]
+  static constexpr size_t nDbl = oBn + (size_t)Mc * NU;
+  static constexpr size_t nInt = 5 * G + 1 + G * kNSten;  // i, pos-valid, u0, nU, prefix[G+1], ok[G][7]
+  static constexpr size_t bytes = nDbl * 8 + nInt * 4 + (size_t)G * kNSten * NE;
+};
+
+template <int M, int GG>
+__global__ void __launch_bounds__(ReconShape<M, GG>::kThreads, 512 / ReconShape<M, GG>::kThreads)
+k_recon_coop(Tab T, Dev d, int initial) {
+  using S = ReconShape<M, GG>;
+  constexpr int Mc = S::Mc, NU = S::NU, NE = S::NE, MaxU = S::MaxU, G = S::G, NL = S::NL, NN = S::NN, RW = S::RW;
+  extern __shared__ double smem[];
+  double* sRow = smem + S::oRow;
+  double* sNrm = smem + S::oNrm;
+  double* sC = smem + S::oC;
+  double* sCh = smem + S::oCh;
+  double* sSig = smem + S::oSig;
+  double* sWc = smem + S::oWc;
+  double* sCv = smem + S::oCv;
+  double* sRL = smem + S::oRL;
+  double* sEl = smem + S::oEl;
+  double* sDt = smem + S::oDt;
+  double* sBn = smem + S::oBn;
+  int* sI = reinterpret_cast<int*>(smem + S::nDbl);
+  int* sVal = sI + G;
+  int* sU0 = sVal + G;
+  int* sNU = sU0 + G;
+  int* sPre = sNU + G;            // G + 1
+  int* sOk = sPre + G + 1;        // G * 7
+  unsigned char* sSt = reinterpret_cast<unsigned char*>(sOk + G * kNSten);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  for (int k = tid; k < Mc * NU; k += nth) sBn[k] = T.Bnod[k / NU][k % NU];
+  const int n_ready = initial ? d.ne : d.cnt->n_ready;
+  const long long Ts = d.cnt->t_sync;
+  for (int consumed = 0; consumed < n_ready;) {
+    // balanced rounds: every block takes the same number of elements (at
+    // most G) per round, so that the elements of the last round spread over
+    // all blocks instead of stacking on a few of them
+    const int per = min(G, (n_ready - consumed + (int)gridDim.x - 1) / (int)gridDim.x);
+    const int base = consumed + (int)blockIdx.x * per;
+    const int cnt = max(0, min(per, n_ready - base));
+    consumed += per * (int)gridDim.x;
+    if (cnt == 0) continue;  // block-uniform
+    // P0: element set-up
+    if (tid < G) {
+      const int e = tid, pos = base + e;
+      const bool v = e < cnt;
+      sVal[e] = v;
+      int nU = 0;
+      if (v) {
+        const int i = initial ? pos : d.ready_list[pos];
+        sI[e] = i;
+        double* el = sEl + e * 16;
+        for (int k = 0; k < 6; ++k) el[k] = d.X[6 * (size_t)i + k];
+        for (int k = 0; k < 4; ++k) el[6 + k] = d.Q[4 * (size_t)i + k];
+        const double ja = el[2] - el[0], jb = el[4] - el[0], jc = el[3] - el[1], jd = el[5] - el[1];
+        const double idet = 1.0 / (ja * jd - jb * jc);
+        el[10] = jd * idet; el[11] = -jb * idet; el[12] = -jc * idet; el[13] = ja * idet;
+        sU0[e] = d.u_ptr[i];
+        nU = d.u_ptr[i + 1] - sU0[e];
+        for (int s = 0; s < kNSten; ++s) sOk[e * kNSten + s] = d.sten_ok[(size_t)i * kNSten + s];
+      }
+      sNU[e] = nU;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      sPre[0] = 0;
+      for (int e = 0; e < G; ++e) sPre[e + 1] = sPre[e] + (sVal[e] ? sNU[e] : 0);
+    }
+    for (int k = tid; k < G * kNSten * NE; k += nth) {
+      const int e = k / (kNSten * NE);
+      sSt[k] = sVal[e] ? d.sten[(size_t)sI[e] * kNSten * NE + k % (kNSten * NE)] : 0;
+    }
+    __syncthreads();
+    // P1: rows of the least-squares systems (virtual data, eqs. virtGeom,
+    // virtCellaverage, intConsRec), then the time-step candidates
+    // (eq. timestep) on the last threads of the block, so that the warps
+    // holding rows do not also run the time-step code with a few lanes
+    for (int item = tid; item < sPre[G]; item += nth) {
+      int e = 0;
+      while (item >= sPre[e + 1]) ++e;
+      const int u = item - sPre[e];
+      const double* el = sEl + e * 16;
+      const long long ti = d.t[sI[e]];
+      double Xv[6], Qv[4];
+      {
+        const int q = sU0[e] + u;
+        const int j = d.u_elem[q];
+        virtual_data<M>(T, d, j, ti, Xv, Qv);
+        const double sx = d.u_shift[2 * (size_t)q], sy = d.u_shift[2 * (size_t)q + 1];
+        double xr[3], yr[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const double px = Xv[2 * k] + sx - el[0], py = Xv[2 * k + 1] + sy - el[1];
+          xr[k] = el[10] * px + el[11] * py - (1.0 / 3.0);
+          yr[k] = el[12] * px + el[13] * py - (1.0 / 3.0);
+        }
+        // averages of the monomials over the virtual member (a straight
+        // triangle) in closed form: with the centroid c and the vertex
+        // offsets u_k = v_k - c, the second central moments are
+        // (1/12) sum_k u_k u_k^T and the third (1/30) sum_k u_k (x) u_k (x) u_k,
+        // so E[x^2] = c_x^2 + S_xx, E[x^2 y] = c_x^2 c_y + c_y S_xx + 2 c_x S_xy
+        // + T_xxy, ...  (what the degree-M quadrature gives, with fewer
+        // operations)
+        double row[NU];
+        const double cx = (xr[0] + xr[1] + xr[2]) * (1.0 / 3.0), cy = (yr[0] + yr[1] + yr[2]) * (1.0 / 3.0);
+        row[0] = cx;
+        row[1] = cy;
+        if constexpr (M >= 2) {
+          double ux[3], uy[3];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            ux[k] = xr[k] - cx;
+            uy[k] = yr[k] - cy;
+          }
+          const double sxx = (ux[0] * ux[0] + ux[1] * ux[1] + ux[2] * ux[2]) * (1.0 / 12.0);
+          const double sxy = (ux[0] * uy[0] + ux[1] * uy[1] + ux[2] * uy[2]) * (1.0 / 12.0);
+          const double syy = (uy[0] * uy[0] + uy[1] * uy[1] + uy[2] * uy[2]) * (1.0 / 12.0);
+          row[2] = cx * cx + sxx;
+          row[3] = cx * cy + sxy;
+          row[4] = cy * cy + syy;
+          if constexpr (M >= 3) {
+            double txxx = 0.0, txxy = 0.0, txyy = 0.0, tyyy = 0.0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const double xx = ux[k] * ux[k], yy = uy[k] * uy[k];
+              txxx += xx * ux[k];
+              txxy += xx * uy[k];
+              txyy += yy * ux[k];
+              tyyy += yy * uy[k];
+            }
+            const double c30 = 1.0 / 30.0;
+            row[5] = cx * (cx * cx + 3.0 * sxx) + txxx * c30;
+            row[6] = cy * (cx * cx + sxx) + 2.0 * cx * sxy + txxy * c30;
+            row[7] = cx * (cy * cy + syy) + 2.0 * cy * sxy + txyy * c30;
+            row[8] = cy * (cy * cy + 3.0 * syy) + tyyy * c30;
+          }
+        }
+        double* dst = sRow + ((size_t)e * (MaxU + 1) + u + 1) * RW;
+#pragma unroll
+        for (int a = 0; a < NU; ++a) dst[a] = row[a] - T.mbar[a];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) dst[NU + v] = Qv[v] - el[6 + v];
+      }
+    }
+    for (int item = nth - 1 - tid; item < G * 4; item += nth) {
+      const int e = item / 4, k = item % 4;
+      if (!sVal[e]) continue;
+      const int i = sI[e];
+      const long long ti = d.t[i];
+      double Xv[6], Qv[4];
+      {
+        const int j = k == 0 ? i : d.nbr[3 * (size_t)i + k - 1];
+        double dtc = DBL_MAX;
+        if (j >= 0 && ti < Ts) {
+          virtual_data<M>(T, d, j, ti, Xv, Qv);
+          double per = 0.0;
+#pragma unroll
+          for (int kk = 0; kk < 3; ++kk) {
+            const int k1 = kk == 2 ? 0 : kk + 1;
+            const double dx = Xv[2 * k1] - Xv[2 * kk], dy = Xv[2 * k1 + 1] - Xv[2 * kk + 1];
+            per += sqrt(dx * dx + dy * dy);
+          }
+          const double dd = 4.0 * area6(Xv) / per;
+          const double uu = Qv[1] / Qv[0], vv = Qv[2] / Qv[0];
+          double vel = sqrt(uu * uu + vv * vv);
+          if (k == 0)  // an element on a moving wall counts the wall's speed
+            for (int e2 = 0; e2 < 3; ++e2)
+              if (d.edge_bc[d.elem_edge[3 * (size_t)i + e2]] == 2) vel = fmax(vel, T.wall_speed);
+          const double lam = vel + sqrt(T.gamma * pressure(T, Qv) / Qv[0]);
+          dtc = (ti < T.Tsw ? T.cfl_start : T.cfl) * dd / lam;
+          if (!(dtc > 0.0)) dtc = -1.0;
+        }
+        sDt[e * 4 + k] = dtc;
+      }
+    }
+    __syncthreads();
+    // P2: normal equations of every stencil
+    for (int item = tid; item < G * kNSten * NN; item += nth) {
+      const int e = item / (kNSten * NN), s = (item / NN) % kNSten, q = item % NN;
+      if (!sVal[e] || !sOk[e * kNSten + s]) continue;
+      int a, b, v = -1;
+      if (q < NL) {
+        a = 0;
+        while ((a + 1) * (a + 2) / 2 <= q) ++a;
+        b = q - a * (a + 1) / 2;
+      } else {
+        a = (q - NL) / 4;
+        v = (q - NL) % 4;
+        b = NU + v;
+      }
+      const unsigned char* st = sSt + (e * kNSten + s) * NE;
+      const double* R0 = sRow + (size_t)e * (MaxU + 1) * RW;
+      double acc = 0.0;
+#pragma unroll
+      for (int m = 1; m < NE; ++m) {
+        const double* r = R0 + (size_t)st[m] * RW;
+        acc += r[a] * r[b];
+      }
+      sNrm[(e * kNSten + s) * NN + q] = acc;
+    }
+    __syncthreads();
+    // P3a: Cholesky factorisation N = L L^T per stencil, in place; the
+    // diagonal keeps 1 / L_aa
+    for (int item = tid; item < G * kNSten; item += nth) {
+      const int e = item / kNSten, s = item % kNSten;
+      if (!sVal[e] || !sOk[e * kNSten + s]) continue;
+      double* nm = sNrm + (size_t)item * NN;
+      double L[NU][NU];
+#pragma unroll
+      for (int a = 0; a < NU; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) L[a][b] = nm[a * (a + 1) / 2 + b];
+#pragma unroll
+      for (int a = 0; a < NU; ++a) {
+        double dd = L[a][a];
+#pragma unroll
+        for (int k = 0; k < a; ++k) dd -= L[a][k] * L[a][k];
+        const double il = rsqrt(dd);
+        L[a][a] = il;
+#pragma unroll
+        for (int b = a + 1; b < NU; ++b) {
+          double v = L[b][a];
+#pragma unroll
+          for (int k = 0; k < a; ++k) v -= L[b][k] * L[a][k];
+          L[b][a] = v * il;
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < NU; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) nm[a * (a + 1) / 2 + b] = L[a][b];
+    }
+    __syncthreads();
+    // P3b: the two triangular solves, one right-hand side per item, then one
+    // step of the corrected semi-normal equations (Bjorck): r = b - A y over
+    // the stencil's rows, solve L L^T dy = A^T r with the same factor,
+    // y += dy.  The normal equations square the condition number of A; the
+    // correction brings y to the accuracy of an orthogonal factorisation.
+    for (int item = tid; item < G * kNSten * 4; item += nth) {
+      const int es = item / 4, v = item % 4, e = es / kNSten, s = es % kNSten;
+      if (!sVal[e] || !sOk[e * kNSten + s]) continue;
+      const double* nm = sNrm + (size_t)es * NN;
+      double* cs = sC + (size_t)es * NU * 4;
+      const unsigned char* st = sSt + es * NE;
+      const double* R0 = sRow + (size_t)e * (MaxU + 1) * RW;
+      double y[NU], z[NU];
+#pragma unroll
+      for (int a = 0; a < NU; ++a) z[a] = nm[NL + a * 4 + v];
+#pragma unroll
+      for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+        for (int a = 0; a < NU; ++a) {
+          double acc = z[a];
+#pragma unroll
+          for (int k = 0; k < a; ++k) acc -= nm[a * (a + 1) / 2 + k] * z[k];
+          z[a] = acc * nm[a * (a + 1) / 2 + a];
+        }
+#pragma unroll
+        for (int a = NU - 1; a >= 0; --a) {
+          double acc = z[a];
+#pragma unroll
+          for (int k = a + 1; k < NU; ++k) acc -= nm[k * (k + 1) / 2 + a] * z[k];
+          z[a] = acc * nm[a * (a + 1) / 2 + a];
+        }
+        if (pass == 0) {
+#pragma unroll
+          for (int a = 0; a < NU; ++a) { y[a] = z[a]; z[a] = 0.0; }
+#pragma unroll
+          for (int m = 1; m < NE; ++m) {
+            const double* r = R0 + (size_t)st[m] * RW;
+            double res = r[NU + v];
+#pragma unroll
+            for (int a = 0; a < NU; ++a) res -= r[a] * y[a];
+#pragma unroll
+            for (int a = 0; a < NU; ++a) z[a] += r[a] * res;
+          }
+        } else {
+#pragma unroll
+          for (int a = 0; a < NU; ++a) y[a] += z[a];
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < NU; ++a) cs[a * 4 + v] = y[a];
+    }
+    __syncthreads();
+    // P4: characteristic fields of dF/dQ.n, n along the density gradient of
+    // the central-stencil polynomial at the centroid (its linear coefficients)
+    if (tid < G && sVal[tid]) {
+      const int e = tid;
+      const double* el = sEl + e * 16;
+      const double* c0 = sC + (size_t)(e * kNSten) * NU * 4;
+      const double gx = c0[0 * 4] * el[10] + c0[1 * 4] * el[12];
+      const double gy = c0[0 * 4] * el[11] + c0[1 * 4] * el[13];
+      // on G lanes of one warp: three reciprocals and two square roots, no
+      // divides (each costs the warp's full FP64 issue)
+      const double gn = sqrt(gx * gx + gy * gy);
+      double nx = 1.0, ny = 0.0;
+      if (gn > 0.0) {
+        const double ign = 1.0 / gn;
+        nx = gx * ign;
+        ny = gy * ign;
+      }
+      const double g = T.gamma, rho = el[6], ir = 1.0 / rho, u = el[7] * ir, v = el[8] * ir;
+      const double p = (g - 1.0) * (el[9] - 0.5 * rho * (u * u + v * v));
+      const double a = sqrt(g * p * ir), H = (el[9] + p) * ir, un = u * nx + v * ny, ut = -u * ny + v * nx;
+      const double ia = 1.0 / a, q2 = 0.5 * (u * u + v * v), b1 = (g - 1.0) * ia * ia, b2 = b1 * q2;
+      double* R = sRL + e * 32;
+      double* Lm = R + 16;
+      R[0] = 1; R[1] = 1; R[2] = 0; R[3] = 1;
+      R[4] = u - a * nx; R[5] = u; R[6] = -ny; R[7] = u + a * nx;
+      R[8] = v - a * ny; R[9] = v; R[10] = nx; R[11] = v + a * ny;
+      R[12] = H - a * un; R[13] = q2; R[14] = ut; R[15] = H + a * un;
+      Lm[0] = 0.5 * (b2 + un * ia); Lm[1] = -0.5 * (b1 * u + nx * ia); Lm[2] = -0.5 * (b1 * v + ny * ia); Lm[3] = 0.5 * b1;
+      Lm[4] = 1.0 - b2; Lm[5] = b1 * u; Lm[6] = b1 * v; Lm[7] = -b1;
+      Lm[8] = -ut; Lm[9] = -ny; Lm[10] = nx; Lm[11] = 0.0;
+      Lm[12] = 0.5 * (b2 - un * ia); Lm[13] = -0.5 * (b1 * u - nx * ia); Lm[14] = -0.5 * (b1 * v - ny * ia); Lm[15] = 0.5 * b1;
+    }
+    __syncthreads();
+    // P5: characteristic coefficients and oscillation indicators (eq. weno)
+    for (int item = tid; item < G * kNSten * 4; item += nth) {
+      const int e = item / (kNSten * 4), s = (item / 4) % kNSten, r = item % 4;
+      if (!sVal[e] || !sOk[e * kNSten + s]) continue;
+      const double* Lr = sRL + e * 32 + 16 + r * 4;
+      const double* cs = sC + (size_t)(e * kNSten + s) * NU * 4;
+      double* ch = sCh + (size_t)(e * kNSten + s) * NU * 4;
+      double cc[NU];
+#pragma unroll
+      for (int l = 0; l < NU; ++l) {
+        cc[l] = Lr[0] * cs[l * 4] + Lr[1] * cs[l * 4 + 1] + Lr[2] * cs[l * 4 + 2] + Lr[3] * cs[l * 4 + 3];
+        ch[l * 4 + r] = cc[l];
+      }
+      double sg = 0.0;
+#pragma unroll
+      for (int a = 0; a < NU; ++a) {
+        double acc = 0.0;
+#pragma unroll
+        for (int b = a; b < NU; ++b) acc += T.SigU[a][b] * cc[b];
+        sg += acc * acc;
+      }
+      sSig[(e * kNSten + s) * 4 + r] = sg;
+    }
+    __syncthreads();
+    // P6: nonlinear weights (one item per element, stencil and field; the
+    // weight overwrites its sigma), then the weighted characteristic
+    // coefficients (one item per element, coefficient and field)
+    for (int item = tid; item < G * kNSten * 4; item += nth) {
+      const int e = item / (kNSten * 4), s = (item / 4) % kNSten;
+      if (!sVal[e]) continue;
+      double om = 0.0;
+      if (sOk[e * kNSten + s]) {
+        const double e1 = sSig[item] + 1e-14;
+        const double e2 = e1 * e1, e4 = e2 * e2, e8 = e4 * e4;
+        om = (s == 0 ? 1e5 : 1.0) / e8;
+      }
+      sSig[item] = om;
+    }
+    __syncthreads();
+    for (int item = tid; item < G * NU * 4; item += nth) {
+      const int e = item / (NU * 4), l = (item / 4) % NU, r = item % 4;
+      if (!sVal[e]) continue;
+      const double* om = sSig + (size_t)e * kNSten * 4 + r;
+      double tot = 0.0;
+#pragma unroll
+      for (int s = 0; s < kNSten; ++s)
+        if (sOk[e * kNSten + s]) tot += om[4 * s];
+      const double itot = 1.0 / tot;
+      double acc = 0.0;
+#pragma unroll
+      for (int s = 0; s < kNSten; ++s)
+        if (sOk[e * kNSten + s]) acc += (om[4 * s] * itot) * sCh[((size_t)(e * kNSten + s) * NU + l) * 4 + r];
+      sWc[(e * NU + l) * 4 + r] = acc;
+    }
+    __syncthreads();
+    // P7: back to conserved variables
+    for (int item = tid; item < G * NU * 4; item += nth) {
+      const int e = item / (NU * 4), l = (item / 4) % NU, v = item % 4;
+      if (!sVal[e]) continue;
+      const double* Rv = sRL + e * 32 + v * 4;
+      const double* wc = sWc + (e * NU + l) * 4;
+      sCv[(e * NU + l) * 4 + v] = Rv[0] * wc[0] + Rv[1] * wc[1] + Rv[2] * wc[2] + Rv[3] * wc[3];
+    }
+    __syncthreads();
+    // P8: nodal values of w_h for the predictor, and the new local time step
+    double* sW0 = sCh;  // free after P6: [G][Mc][4]
+    for (int item = tid; item < G * (Mc * 4 + 1); item += nth) {
+      const int e = item / (Mc * 4 + 1), k = item % (Mc * 4 + 1);
+      if (!sVal[e]) continue;
+      const int i = sI[e];
+      if (k < Mc * 4) {
+        const int s = k / 4, v = k % 4;
+        double acc = sEl[e * 16 + 6 + v];
+#pragma unroll
+        for (int l = 0; l < NU; ++l) acc += sBn[s * NU + l] * sCv[(e * NU + l) * 4 + v];
+        sW0[(e * Mc + s) * 4 + v] = acc;
+      } else {
+        const long long ti = d.t[i];
+        long long tks = 0;
+        if (ti < Ts) {
+          double best = DBL_MAX;
+          bool bad = false;
+          for (int c = 0; c < 4; ++c) {
+            const double v = sDt[e * 4 + c];
+            if (v < 0.0) bad = true;
+            best = fmin(best, v);
+          }
+          if (bad || !(best > 0.0)) {
+            set_error(d.cnt, -3, i);
+            best = d.etick[i];
+          }
+          const double rt = floor(best / d.etick[i]);
+          const bool start = ti < T.Tsw;  // global-step start-up
+          const long long end = start ? (T.Tsw < Ts ? T.Tsw : Ts) : Ts;
+          tks = rt > (double)(end - ti) ? end - ti : (long long)rt;
+          if (tks < 1) tks = 1;
+          if (T.gts || start) atomicMin(&d.cnt->gts_min, tks);
+        }
+        if (d.sched_mode) {  // frozen schedule: record or replay this update's step
+          const long long ci = d.count[i];
+          if (ci >= d.sched_k) {
+            set_error(d.cnt, -7, i);
+          } else {
+            long long* slot = d.sched_log + (size_t)i * d.sched_k + ci;
+            if (d.sched_mode == 1) *slot = tks;
+            else tks = *slot;
+          }
+        }
+        d.dt[i] = tks;
+      }
+    }
+    __syncthreads();
+    // P9: positivity scaling of w_h at the lattice nodes (density first, then
+    // pressure through its chord bound; the scaling of Zhang and Shu), then
+    // the nodal values go to the predictor.  Per pass: one candidate theta per
+    // node, the element's minimum, the scaling.
+    for (int pass = 0; pass < 2; ++pass) {
+      double* cand = sSig;  // [G][Mc], free after P6
+      for (int item = tid; item < G * Mc; item += nth) {
+        const int e = item / Mc;
+        if (!sVal[e]) continue;
+        const double* Qi = sEl + e * 16 + 6;
+        const double* ws = sW0 + (size_t)item * 4;
+        double th = 1.0;
+        if (pass == 0) {
+          const double rho_min = 1e-8 * Qi[0];
+          if (ws[0] < rho_min) th = (Qi[0] - rho_min) / (Qi[0] - ws[0]);
+        } else {
+          const double p_i = pressure(T, Qi), p_min = 1e-8 * p_i, ps = pressure(T, ws);
+          if (ps < p_min) th = (p_i - p_min) / (p_i - ps);
+        }
+        cand[item] = th;
+      }
+      __syncthreads();
+      for (int e = tid; e < G; e += nth) {
+        double theta = 1.0;
+        if (sVal[e])
+          for (int k = 0; k < Mc; ++k) theta = fmin(theta, cand[e * Mc + k]);
+        sDt[e * 4] = theta;  // free after P8
+      }
+      __syncthreads();
+      for (int item = tid; item < G * Mc * 4; item += nth) {
+        const int e = item / (Mc * 4);
+        const double theta = sDt[e * 4];
+        if (!sVal[e] || !(theta < 1.0)) continue;
+        const double qi = sEl[e * 16 + 6 + item % 4];
+        sW0[item] = qi + theta * (sW0[item] - qi);
+      }
+      __syncthreads();
+    }
+    for (int item = tid; item < G * Mc * 4; item += nth) {
+      const int e = item / (Mc * 4);
+      if (!sVal[e]) continue;
+      d.w0[(size_t)(base + e) * Mc * 4 + item % (Mc * 4)] = sW0[item];
+    }
+    __syncthreads();
+  }
+}
+
+// The reconstruction and predictor grids cover every element (the pre-
+// processing phase) or bpsm blocks per SM that loop over the ready list.
+template <int M, int GG>
+void launch_recon_g(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, int bpsm) {
+  using S = ReconShape<M, GG>;
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_recon_coop<M, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::bytes);
+    attr = true;
+  }
+  const int need = (d.ne + S::G - 1) / S::G;
+  const int grid = initial ? need : std::min(need, nsm * bpsm);
+  k_recon_coop<M, GG><<<grid, S::kThreads, S::bytes, s>>>(T, d, initial);
+}
+
+template <int M>
+void launch_recon(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl) {
+  constexpr int G0 = recon_g_default<M>();
+  if (tl.recon_half) launch_recon_g<M, G0 / 2>(T, d, nsm, s, initial, tl.bpsm);
+  else launch_recon_g<M, G0>(T, d, nsm, s, initial, tl.bpsm);
+}
+
 template <int M, int TH>
 void launch_predict_t(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, int bpsm) {
   using S = PredShape<M, TH>;
@@ -335,6 +912,14 @@ void launch_predict(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int ini
 }
 
 }  // namespace
+
+void launch_plain_recon(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl) {
+  switch (T.M) {
+    case 1: launch_recon<1>(T, d, nsm, s, initial, tl); break;
+    case 2: launch_recon<2>(T, d, nsm, s, initial, tl); break;
+    default: launch_recon<3>(T, d, nsm, s, initial, tl); break;
+  }
+}
 
 void launch_plain_predict(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl) {
   switch (T.M) {

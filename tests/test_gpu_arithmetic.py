@@ -35,6 +35,34 @@ __global__ void k_limbs(const double* x, const int* E, float4* f, double* j, int
     j[i] = aw::join18(f[i].x, f[i].y, f[i].z) * aw::limb_unit(E[i]);
   }
 }
+__global__ void k_roots(const double* x, double* s, double* r, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) {
+    s[i] = aw::sqrt5(x[i]);
+    r[i] = aw::rsqrt5(x[i]);
+  }
+}
+// one dot product of `len` terms per thread, as the least-squares sums take it
+__global__ void k_dot(const double* a, const double* b, int len, long long* hh, long long* hl, float2* f, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  long long h = 0, l = 0;
+  for (int k = 0; k < len; ++k)
+    aw::dot28(h, l, aw::limbs28(aw::fixed_point<57>(a[i * len + k], 1022)),
+              aw::limbs28(aw::fixed_point<57>(b[i * len + k], 1022)));
+  hh[i] = h;
+  hl[i] = l;
+  const aw::F2 g = aw::f2_of_dot(h, l);
+  f[i] = make_float2(g.h, g.l);
+}
+extern "C" int roots(const double* x, double* s, double* r, int n) {
+  k_roots<<<(n + 127) / 128, 128>>>(x, s, r, n);
+  return cudaDeviceSynchronize();
+}
+extern "C" int dot(const double* a, const double* b, int len, long long* hh, long long* hl, float2* f, int n) {
+  k_dot<<<(n + 127) / 128, 128>>>(a, b, len, hh, hl, f, n);
+  return cudaDeviceSynchronize();
+}
 extern "C" int rcp(const double* x, double* y, int n) {
   k_rcp<<<(n + 127) / 128, 128>>>(x, y, n);
   return cudaDeviceSynchronize();
@@ -69,6 +97,45 @@ def test_reciprocal(lib):
     assert lib.rcp(_p(xd), _p(y), x.size) == 0
     y, r = y.cpu().numpy(), 1.0 / x
     assert (np.abs(y - r) <= np.spacing(np.abs(r))).all()
+
+
+def test_roots(lib):
+    """sqrt and its reciprocal from series truncated below 2^-60 with at most
+    three roundings of half an ulp on small terms or halved: one ulp; zero and
+    subnormal arguments of the square root give 0, negative ones NaN."""
+    rng = np.random.default_rng(3)
+    x = np.ldexp(rng.uniform(1.0, 2.0, 200000), rng.integers(-1020, 1020, 200000))
+    x[:6] = 1.0, 4.0, np.nextafter(4.0, 5.0), 0.0, 1e-310, -1.0
+    xd = torch.tensor(x, device="cuda")
+    s, r = torch.empty_like(xd), torch.empty_like(xd)
+    assert lib.roots(_p(xd), _p(s), _p(r), x.size) == 0
+    s, r = s.cpu().numpy(), r.cpu().numpy()
+    assert s[3] == 0.0 and s[4] == 0.0 and np.isnan(s[5])
+    k = np.r_[0:3, 6:x.size]
+    assert (np.abs(s[k] - np.sqrt(x[k])) <= np.spacing(np.sqrt(x[k]))).all()
+    ref = (1.0 / np.sqrt(x[k].astype(np.longdouble))).astype(np.float64)
+    assert (np.abs(r[k] - ref) <= 1.5 * np.spacing(ref)).all()
+
+
+@pytest.mark.parametrize("length", [1, 11, 19])
+def test_integer_dot(lib, length):
+    """hh 2^28 + hl equals the product sum but for the low limbs' products,
+    which are below 2^54 each; the pair of floats carries 46 bits of it."""
+    rng = np.random.default_rng(4)
+    n = 3000
+    a, b = (np.ldexp(rng.uniform(-0.5, 0.5, (n, length)), -rng.integers(0, 30, (n, length))) for _ in range(2))
+    ad, bd = torch.tensor(a, device="cuda"), torch.tensor(b, device="cuda")
+    hh, hl = (torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(2))
+    f = torch.empty((n, 2), dtype=torch.float32, device="cuda")
+    assert lib.dot(_p(ad), _p(bd), length, _p(hh), _p(hl), _p(f), n) == 0
+    hh, hl, f = hh.cpu().numpy(), hl.cpu().numpy(), f.cpu().numpy().astype(np.float64)
+    half_up = lambda v: int(np.floor(abs(v) * 2.0 ** 57 + 0.5)) * (1 if v >= 0 else -1)  # noqa: E731
+    for i in range(n):
+        exact = sum(half_up(x) * half_up(y) for x, y in zip(a[i], b[i]))
+        got = (int(hh[i]) << 56) + (int(hl[i]) << 28)
+        assert abs(got - exact) <= length << 54, i
+        v = got / 2.0 ** 56
+        assert abs(f[i, 0] + f[i, 1] - v) <= abs(v) * 2.0 ** -46 + 2.0 ** -20, i
 
 
 def test_limbs(lib):

@@ -19,6 +19,8 @@ namespace aw {
 
 namespace {
 
+constexpr int kBlock = 128;
+
 __device__ __forceinline__ double area6(const double* X) {
   return 0.5 * ((X[2] - X[0]) * (X[5] - X[1]) - (X[3] - X[1]) * (X[4] - X[0]));
 }
@@ -29,6 +31,286 @@ __device__ __forceinline__ void set_error(Counters* cnt, int code, int elem) {
 
 __device__ __forceinline__ double pressure(const Tab& T, const double* q) {
   return (T.gamma - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
+}
+
+// Exact state of the Kidder compression (Sec. 3.4, eqs. KidderIC, KidderEx)
+// at (x, y, t): a particle starting at radius r sits at h(t) r with
+// h = sqrt(1 - t^2/tau^2); density rho0(r)/h^2 with rho0^(gamma-1) linear in
+// r^2 between the two frontiers, radial velocity h' r, pressure s0 rho^gamma;
+// tau = sqrt((gamma-1)/2 (r_e0^2 - r_i0^2)/(c_e0^2 - c_i0^2)).
+__device__ void kidder_state(const Tab& T, double x, double y, double t, double* q) {
+  const double g = T.gamma, ri = T.kidder[0], re = T.kidder[1], s0 = T.kidder[4];
+  const double ai = pow(T.kidder[2], g - 1.0), ae = pow(T.kidder[3], g - 1.0);
+  const double ci2 = g * s0 * ai, ce2 = g * s0 * ae;
+  const double tau2 = 0.5 * (g - 1.0) * (re * re - ri * ri) / (ce2 - ci2);
+  const double h = sqrt(1.0 - t * t / tau2), dh = -t / (tau2 * h);
+  const double R = sqrt(x * x + y * y), r = R / h;
+  const double w = (r * r - ri * ri) / (re * re - ri * ri);
+  const double rho = pow((1.0 - w) * ai + w * ae, 1.0 / (g - 1.0)) / (h * h);
+  const double u = dh / h * x, v = dh / h * y;
+  const double p = s0 * pow(rho, g);
+  q[0] = rho;
+  q[1] = rho * u;
+  q[2] = rho * v;
+  q[3] = p / (g - 1.0) + 0.5 * rho * (u * u + v * v);
+}
+
+// Rusanov-type ALE flux through the area-weighted space-time normal n
+// (eq. rusanov): the largest |eigenvalue| of A_n^V times |n_xy| is
+// |v.n_xy + n_t| + c |n_xy|.
+__device__ __forceinline__ void rusanov(const Tab& T, const double* qm, const double* qp, const double* n,
+                                        double* F) {
+  // both sides' 1 / rho from one reciprocal
+  const double rr = 1.0 / (qm[0] * qp[0]);
+  double rim = qp[0] * rr, rip = qm[0] * rr;
+  double um = qm[1] * rim, vm = qm[2] * rim, up = qp[1] * rip, vp = qp[2] * rip;
+  double pm = (T.gamma - 1.0) * (qm[3] - 0.5 * (qm[1] * um + qm[2] * vm));
+  double pp = (T.gamma - 1.0) * (qp[3] - 0.5 * (qp[1] * up + qp[2] * vp));
+  // c |n_xy| as one square root per side
+  double nn2 = n[0] * n[0] + n[1] * n[1];
+  double cmn = sqrt(T.gamma * pm * rim * nn2), cpn = sqrt(T.gamma * pp * rip * nn2);
+  double wm = um * n[0] + vm * n[1] + n[2], wp = up * n[0] + vp * n[1] + n[2];
+  double sm = fabs(wm) + cmn, sp = fabs(wp) + cpn;
+  double smax = fmax(sm, sp);
+  // F~.n = f n_x + g n_y + q n_t = q (v.n_xy + n_t) + p (0, n_x, n_y, v.n_xy)
+  double vnm = um * n[0] + vm * n[1], vnp = up * n[0] + vp * n[1];
+  double Fm[4] = {qm[0] * wm, qm[1] * wm + pm * n[0], qm[2] * wm + pm * n[1], qm[3] * wm + pm * vnm};
+  double Fp[4] = {qp[0] * wp, qp[1] * wp + pp * n[0], qp[2] * wp + pp * n[1], qp[3] * wp + pp * vnp};
+#pragma unroll
+  for (int v = 0; v < 4; ++v) F[v] = 0.5 * (Fm[v] + Fp[v]) - 0.5 * smax * (qp[v] - qm[v]);
+}
+
+// Osher-type ALE flux (eq. osher) on the straight path Psi(s) = q- + s (q+ -
+// q-) (eq. path), the path integral by 3-point Gauss-Legendre quadrature:
+// at each path node |A| dq = R |Lambda| L dq with the eigenvalues
+// |n_xy| (u_n - c, u_n, u_n, u_n + c) + n_t of the ALE Jacobian and the
+// eigenvectors R, L = R^-1 of dF/dQ.n, n = n_xy / |n_xy|.
+__device__ __forceinline__ void osher(const Tab& T, const double* qm, const double* qp, const double* n,
+                                      double* F) {
+  const double g = T.gamma, gm1 = g - 1.0;
+  double rim = 1.0 / qm[0], rip = 1.0 / qp[0];
+  double um = qm[1] * rim, vm = qm[2] * rim, up = qp[1] * rip, vp = qp[2] * rip;
+  double pm = gm1 * (qm[3] - 0.5 * (qm[1] * um + qm[2] * vm));
+  double pp = gm1 * (qp[3] - 0.5 * (qp[1] * up + qp[2] * vp));
+  double wm = um * n[0] + vm * n[1] + n[2], wp = up * n[0] + vp * n[1] + n[2];
+  double vnm = um * n[0] + vm * n[1], vnp = up * n[0] + vp * n[1];
+  const double nxy = sqrt(n[0] * n[0] + n[1] * n[1]);
+  double nx = 1.0, ny = 0.0;
+  if (nxy > 0.0) {
+    const double inx = 1.0 / nxy;
+    nx = n[0] * inx;
+    ny = n[1] * inx;
+  }
+  double dq[4], D[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int v = 0; v < 4; ++v) dq[v] = qp[v] - qm[v];
+  const double r15 = 0.38729833462074168852;  // sqrt(15) / 10
+#pragma unroll
+  for (int gq = 0; gq < 3; ++gq) {
+    const double s = gq == 0 ? 0.5 - r15 : (gq == 1 ? 0.5 : 0.5 + r15);
+    const double ws = gq == 1 ? 8.0 / 18.0 : 5.0 / 18.0;
+    double q[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) q[v] = qm[v] + s * dq[v];
+    const double ir = 1.0 / q[0], u = q[1] * ir, v = q[2] * ir;
+    const double p = gm1 * (q[3] - 0.5 * (q[1] * u + q[2] * v));
+    const double a = sqrt(g * p * ir), ia = 1.0 / a, H = (q[3] + p) * ir;
+    const double un = u * nx + v * ny, ut = -u * ny + v * nx, q2 = 0.5 * (u * u + v * v);
+    const double b1 = gm1 * ia * ia, b2 = b1 * q2;
+    // characteristic amplitudes L dq, scaled by |lambda|
+    double c0 = 0.5 * (b2 + un * ia) * dq[0] - 0.5 * (b1 * u + nx * ia) * dq[1] - 0.5 * (b1 * v + ny * ia) * dq[2] +
+                0.5 * b1 * dq[3];
+    double c1 = (1.0 - b2) * dq[0] + b1 * u * dq[1] + b1 * v * dq[2] - b1 * dq[3];
+    double c2 = -ut * dq[0] - ny * dq[1] + nx * dq[2];
+    double c3 = 0.5 * (b2 - un * ia) * dq[0] - 0.5 * (b1 * u - nx * ia) * dq[1] - 0.5 * (b1 * v - ny * ia) * dq[2] +
+                0.5 * b1 * dq[3];
+    c0 *= ws * fabs(nxy * (un - a) + n[2]);
+    c1 *= ws * fabs(nxy * un + n[2]);
+    c2 *= ws * fabs(nxy * un + n[2]);
+    c3 *= ws * fabs(nxy * (un + a) + n[2]);
+    D[0] += c0 + c1 + c3;
+    D[1] += (u - a * nx) * c0 + u * c1 - ny * c2 + (u + a * nx) * c3;
+    D[2] += (v - a * ny) * c0 + v * c1 + nx * c2 + (v + a * ny) * c3;
+    D[3] += (H - a * un) * c0 + q2 * c1 + ut * c2 + (H + a * un) * c3;
+  }
+  const double Fm[4] = {qm[0] * wm, qm[1] * wm + pm * n[0], qm[2] * wm + pm * n[1], qm[3] * wm + pm * vnm};
+  const double Fp[4] = {qp[0] * wp, qp[1] * wp + pp * n[0], qp[2] * wp + pp * n[1], qp[3] * wp + pp * vnp};
+#pragma unroll
+  for (int v = 0; v < 4; ++v) F[v] = 0.5 * (Fm[v] + Fp[v]) - 0.5 * D[v];
+}
+
+// Per-edge data of a swept surface, formed once per edge (not once per Gauss
+// point): its four corners (x, y, t in seconds: a, b at the old node times,
+// b', a' at the new ones), the corner ticks, and for each side its element,
+// local edge, time (ticks) and reciprocal step (0 for a zero step).
+struct EdgeSetup {
+  double P[4][3];
+  double tk[4];
+  double tL, itL, tR, itR, etL;
+  int L, R, le, lr, bc;
+};
+
+// One lane per Gauss point: (M+1)^2 consecutive lanes per swept edge,
+// 32 / (M+1)^2 edges per warp, the point contributions summed by a fixed
+// shuffle tree within each edge's lanes.
+template <int M>
+__global__ void __launch_bounds__(kBlock) k_flux_grp(Tab T, Dev d) {
+  // one thread per Gauss point, the block's EPB edges packed back to back
+  // (an edge's points may span two warps: every lane of a warp FP64
+  // instruction costs the pipe the same, used or not), the point sums
+  // through shared memory in point order.  The per-edge set-up runs first,
+  // one thread per edge, so that its FP64 work (tick conversions, the
+  // sides' reciprocal steps) is issued once per edge instead of once per
+  // Gauss point.
+  constexpr int Nt = M + 1, NP = Nt * Nt, EPB = kBlock / NP;
+  __shared__ double sGN[kBlock][7];
+  __shared__ EdgeSetup sE[EPB];
+  const int epoch = d.cnt->epoch;
+  const int n_active = d.cnt->n_active;
+  const int slot = threadIdx.x / NP, pt = threadIdx.x % NP;
+  for (int first = blockIdx.x * EPB; first < n_active; first += gridDim.x * EPB) {
+    for (int k = threadIdx.x; k < EPB; k += kBlock) {
+      if (first + k >= n_active) continue;
+      const int ed = d.active_list[first + k];
+      const int a = d.edge_nodes[2 * ed], b = d.edge_nodes[2 * ed + 1];
+      const int L = d.edge_elem[2 * ed], R = d.edge_elem[2 * ed + 1];
+      const int le = d.edge_loc[2 * ed], lr = d.edge_loc[2 * ed + 1];
+      const bool ma = d.node_moved[a] == epoch, mb = d.node_moved[b] == epoch;
+      const int le1 = le == 2 ? 0 : le + 1;
+      const double sax = d.cshift[6 * L + 2 * le], say = d.cshift[6 * L + 2 * le + 1];
+      const double sbx = d.cshift[6 * L + 2 * le1], sby = d.cshift[6 * L + 2 * le1 + 1];
+      const long long tL = d.t[L], dtL = d.dt[L];
+      const double etL = d.etick[L];
+      long long tR = 0, dtR = 0;
+      if (R >= 0) {
+        tR = d.t[R];
+        dtR = d.dt[R];
+      }
+      EdgeSetup& E = sE[k];
+      long long tk[4];
+      E.P[0][0] = d.nX[2 * a] + sax; E.P[0][1] = d.nX[2 * a + 1] + say; tk[0] = d.nt[a];
+      E.P[1][0] = d.nX[2 * b] + sbx; E.P[1][1] = d.nX[2 * b + 1] + sby; tk[1] = d.nt[b];
+      if (mb) { E.P[2][0] = d.nXn[2 * b] + sbx; E.P[2][1] = d.nXn[2 * b + 1] + sby; tk[2] = d.ntn[b]; }
+      else { E.P[2][0] = E.P[1][0]; E.P[2][1] = E.P[1][1]; tk[2] = tk[1]; }
+      if (ma) { E.P[3][0] = d.nXn[2 * a] + sax; E.P[3][1] = d.nXn[2 * a + 1] + say; tk[3] = d.ntn[a]; }
+      else { E.P[3][0] = E.P[0][0]; E.P[3][1] = E.P[0][1]; tk[3] = tk[0]; }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        E.tk[c] = (double)tk[c];
+        E.P[c][2] = E.tk[c] * etL;
+      }
+      // a reciprocal costs the FP64 pipe half a divide
+      E.tL = (double)tL;
+      E.itL = dtL > 0 ? 1.0 / (double)dtL : 0.0;
+      E.tR = (double)tR;
+      E.itR = dtR > 0 ? 1.0 / (double)dtR : 0.0;
+      E.etL = etL;
+      E.L = L; E.R = R; E.le = le; E.lr = lr;
+      E.bc = d.edge_bc[ed];
+    }
+    __syncthreads();
+    const int q = first + slot;
+    const bool valid = slot < EPB && q < n_active;
+    double G[4] = {0, 0, 0, 0}, Nn[3] = {0, 0, 0};
+    if (valid) {
+      const EdgeSetup& E = sE[slot];
+      const int gx = pt / Nt, gt = pt % Nt;
+      const int L = E.L, R = E.R, le = E.le, lr = E.lr;
+      double P[4][3];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) P[k][c] = E.P[k][c];
+      const double chi = T.glx[gx], tau = T.glx[gt], wq = T.glw[gx] * T.glw[gt];
+      double dchi[3], dtau[3], n[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        dchi[c] = (1.0 - tau) * (P[1][c] - P[0][c]) + tau * (P[2][c] - P[3][c]);
+        dtau[c] = (1.0 - chi) * (P[3][c] - P[0][c]) + chi * (P[2][c] - P[1][c]);
+      }
+      n[0] = dchi[1] * dtau[2] - dchi[2] * dtau[1];
+      n[1] = dchi[2] * dtau[0] - dchi[0] * dtau[2];
+      n[2] = dchi[0] * dtau[1] - dchi[1] * dtau[0];
+      const double tt = (1 - chi) * (1 - tau) * E.tk[0] + chi * (1 - tau) * E.tk[1] + chi * tau * E.tk[2] +
+                        (1 - chi) * tau * E.tk[3];
+      double qm[4], qp[4];
+      {
+        const double tl = (tt - E.tL) * E.itL;
+        const double* c0 = d.trace + ((((size_t)L * 3 + le) * Nt + gx) * Nt) * 4;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          double acc = c0[(Nt - 1) * 4 + v];
+#pragma unroll
+          for (int p = Nt - 2; p >= 0; --p) acc = acc * tl + c0[p * 4 + v];
+          qm[v] = acc;
+        }
+      }
+      const int bc = E.bc;
+      if (R >= 0) {
+        const double tr = (tt - E.tR) * E.itR;
+        const double* c0 = d.trace + ((((size_t)R * 3 + lr) * Nt + (Nt - 1 - gx)) * Nt) * 4;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          double acc = c0[(Nt - 1) * 4 + v];
+#pragma unroll
+          for (int p = Nt - 2; p >= 0; --p) acc = acc * tr + c0[p * 4 + v];
+          qp[v] = acc;
+        }
+      } else if (bc == 1) {
+        // transmissive: the boundary element's sweep-start average (phase A
+        // updates Q after this kernel), not the inner trace value, with
+        // which a gas at rest beside the boundary grows from roundoff
+#pragma unroll
+        for (int v = 0; v < 4; ++v) qp[v] = d.Q[4 * (size_t)L + v];
+      } else if (bc == 3) {
+        // the exact Kidder state at the quadrature point
+        const double px = (1 - chi) * (1 - tau) * P[0][0] + chi * (1 - tau) * P[1][0] + chi * tau * P[2][0] +
+                          (1 - chi) * tau * P[3][0];
+        const double py = (1 - chi) * (1 - tau) * P[0][1] + chi * (1 - tau) * P[1][1] + chi * tau * P[2][1] +
+                          (1 - chi) * tau * P[3][1];
+        kidder_state(T, px, py, tt * E.etL, qp);
+      } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) qp[v] = qm[v];
+        if (bc == 0 || bc == 2) {  // mirror the normal momentum relative to the wall
+          const double wu = bc == 2 ? T.wall_u : 0.0, wv = bc == 2 ? T.wall_v : 0.0;
+          const double nn = n[0] * n[0] + n[1] * n[1];
+          if (nn > 0.0) {
+            const double mn = ((qm[1] - qm[0] * wu) * n[0] + (qm[2] - qm[0] * wv) * n[1]) / nn;
+            qp[1] = qm[1] - 2.0 * mn * n[0];
+            qp[2] = qm[2] - 2.0 * mn * n[1];
+            // same internal energy: a moving wall's mirror changes the kinetic energy
+            if (bc == 2)
+              qp[3] = qm[3] + 0.5 * (qp[1] * qp[1] + qp[2] * qp[2] - qm[1] * qm[1] - qm[2] * qm[2]) / qm[0];
+          }
+        }
+      }
+      double F[4];
+      if (T.flux == 1) osher(T, qm, qp, n, F);
+      else rusanov(T, qm, qp, n, F);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) G[v] = wq * F[v];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) Nn[c] = wq * n[c];
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) sGN[threadIdx.x][v] = G[v];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sGN[threadIdx.x][4 + c] = Nn[c];
+    __syncthreads();
+    // one thread per (edge, component): the flux G (4) and the GCL vector (3)
+    for (int it = threadIdx.x; it < EPB * 7; it += kBlock) {
+      const int le = it / 7, k = it % 7, qq = first + le;
+      if (qq >= n_active) continue;
+      double acc = sGN[le * NP][k];
+#pragma unroll
+      for (int p2 = 1; p2 < NP; ++p2) acc += sGN[le * NP + p2][k];
+      const int e2 = d.active_list[qq];
+      if (k < 4) d.G[4 * (size_t)e2 + k] = acc;
+      else d.N[4 * (size_t)e2 + k - 4] = acc;
+    }
+    __syncthreads();
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -912,6 +1194,15 @@ void launch_predict(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int ini
 }
 
 }  // namespace
+
+void launch_plain_flux(const Tab& T, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl) {
+  const int grid = nsm * tl.bpsm * 4;
+  switch (T.M) {
+    case 1: k_flux_grp<1><<<grid, kBlock, 0, s>>>(T, d); break;
+    case 2: k_flux_grp<2><<<grid, kBlock, 0, s>>>(T, d); break;
+    default: k_flux_grp<3><<<grid, kBlock, 0, s>>>(T, d); break;
+  }
+}
 
 void launch_plain_recon(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl) {
   switch (T.M) {

@@ -31,10 +31,6 @@ struct aw_ctx {
   bool prof = false;         // per-kernel CUDA-event timing of sweeps
   cudaGraphExec_t prof_graph[2] = {};  // the sweep with an event before and after every kernel
   cudaEvent_t prof_ev[kNumKernels + 1] = {};
-  // side stream of the sweep graph: the node solver runs beside the edge
-  // marking (they read the moved-node list and write disjoint arrays)
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   double prof_ms[kNumKernels] = {0};
   long long prof_sweeps = 0;
   long long ne = 0, nn = 0, ned = 0, sw_total = 0, u_total = 0;
@@ -42,6 +38,7 @@ struct aw_ctx {
   double* d_corner0 = nullptr;  // element corners at t = 0
   std::vector<double> etick_h, ntick_h;  // seconds per tick of each element / node
   cudaGraphExec_t graph_exec[2] = {};  // one captured sweep: the fast and the plain kernels (Dev::plain)
+  cudaGraphExec_t graph_run[2] = {};   // kRun captured sweeps
   Tiles tiles;                           // tile shapes of the sweep kernels
   std::vector<int> tri_h;                // host copies for aw_load_state_xy
   std::vector<double> cshift_h;
@@ -662,6 +659,8 @@ int dupload(aw_ctx* c, const T** out, const std::vector<T>& v) {
 void drop_graphs(aw_ctx* c) {
   for (int k = 0; k < 2; ++k) {
     if (c->graph_exec[k]) cudaGraphExecDestroy(c->graph_exec[k]);
+    if (c->graph_run[k]) cudaGraphExecDestroy(c->graph_run[k]);
+    c->graph_run[k] = nullptr;
     if (c->prof_graph[k]) cudaGraphExecDestroy(c->prof_graph[k]);
     c->graph_exec[k] = c->prof_graph[k] = nullptr;
   }
@@ -872,9 +871,6 @@ void aw_destroy(aw_ctx* c) {
   free_all(c);
   for (cudaEvent_t e : c->prof_ev)
     if (e) cudaEventDestroy(e);
-  if (c->fork_ev) cudaEventDestroy(c->fork_ev);
-  if (c->join_ev) cudaEventDestroy(c->join_ev);
-  if (c->side) cudaStreamDestroy(c->side);
   if (c->hcnt) cudaFreeHost(c->hcnt);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
@@ -1109,21 +1105,26 @@ static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
   // With profiling it is a second graph with an event record between the
   // kernels: each profiled sweep waits for its last event and adds the
   // kernel times (the kernels run as in the plain graph).
+  // A run of kRun sweeps is one graph, so that the gap between two graph
+  // launches is paid once per run (captured when a call first asks for as many).
+  // Sweeps with nothing to do: 12.3 us each in graphs of one, 9.2 of four, 9.0 of eight.
+  constexpr int kRun = 4;
   cudaGraphExec_t& graph = c->graph_exec[c->d.plain];
+  cudaGraphExec_t& run = c->graph_run[c->d.plain];
   cudaGraphExec_t& prof_graph = c->prof_graph[c->d.plain];
-  if (!c->prof && !graph) {
-    if (!c->side) {
-      CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-      CK(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
-      CK(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
-    }
+  auto capture = [&](cudaGraphExec_t& exec, int sweeps) -> int {
     cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    launch_sweep(c->tab, c->d, c->nsm, c->stream, nullptr, c->tiles, c->side, c->fork_ev, c->join_ev);
+    for (int k = 0; k < sweeps; ++k) launch_sweep(c->tab, c->d, c->nsm, c->stream, nullptr, c->tiles);
     CK(cudaStreamEndCapture(c->stream, &g));
-    CK(cudaGraphInstantiate(&graph, g, 0));
+    const cudaError_t e = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
-  }
+    CK(e);
+    return AW_OK;
+  };
+  int rcg = AW_OK;
+  if (!c->prof && !graph && (n % kRun != 0 || n == 0) && (rcg = capture(graph, 1))) return rcg;
+  if (!c->prof && !run && n >= kRun && (rcg = capture(run, kRun))) return rcg;
   if (c->prof && !prof_graph) {
     for (cudaEvent_t& e : c->prof_ev)
       if (!e) CK(cudaEventCreate(&e));
@@ -1144,6 +1145,9 @@ static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
         c->prof_ms[q] += ms;
       }
       c->prof_sweeps += 1;
+    } else if (n - k >= kRun) {
+      CK(cudaGraphLaunch(run, c->stream));
+      k += kRun - 1;
     } else {
       CK(cudaGraphLaunch(graph, c->stream));
     }

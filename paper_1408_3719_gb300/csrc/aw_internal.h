@@ -184,12 +184,9 @@ struct Tiles {
 };
 
 // kernel launchers (aw_kernels.cu)
-constexpr int kNumKernels = 8;  // launches per sweep
+constexpr int kNumKernels = 7;  // timed parts of a sweep (k_finish: plain kernels only)
 const char* kernel_name(int k);
-// side, fork, join (optional, plain launches only): the node solver on the
-// side stream, beside the edge marking on s
-void launch_sweep(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, cudaEvent_t* ev, const Tiles& tl,
-                  cudaStream_t side = nullptr, cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
+void launch_sweep(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, cudaEvent_t* ev, const Tiles& tl);
 void launch_initial(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl);
 void launch_products(const Tab& tab, const Dev& d, int nsm, cudaStream_t s);
 // a new sync time Tn below the current one: every step crossing Tn is cut back
@@ -203,7 +200,7 @@ void launch_plain_flux(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, co
 void launch_plain_recon(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 void launch_plain_predict(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 double measure_fp64_peak();
-// k_ready, k_nodes, k_edges of one sweep: ready/moved/active/touched lists
+// k_ready and k_nodes_edges of one sweep: ready/moved/active/touched lists
 // and the new node positions, without changing the state
 void launch_phase_a_lists(const Tab& tab, const Dev& d, int nsm, cudaStream_t s);
 

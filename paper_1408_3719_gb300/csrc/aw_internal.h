@@ -197,6 +197,7 @@ void launch_sync_cut(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long
 void launch_sync_resume(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, long long Told, const Tiles& tl);
 // the same kernels' plain FP64 forms (aw_plain.cu)
 void launch_plain_flux(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl);
+void launch_plain_update(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl);
 void launch_plain_recon(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 void launch_plain_predict(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl);
 double measure_fp64_peak();

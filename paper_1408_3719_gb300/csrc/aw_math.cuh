@@ -82,12 +82,25 @@ __device__ __forceinline__ double limb_unit(int E) {
   return E >= 0x7ff ? __longlong_as_double(0x7ff8000000000000LL) : __hiloint2double((E - 53) << 20, 0);
 }
 
+// (double)q for |q| <= 2^62 on the integer pipes, the same to the bit: the
+// conversion instruction takes the FP64 pipe's 16 SM cycles, these two dozen
+// about 10, though more time from end to end
+__device__ __forceinline__ double int_to_double(long long q) {
+  const unsigned long long a = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << ((lz - 1) & 63);  // 2^62 <= m < 2^63
+  const unsigned long long r = (m + 0x1ff + ((m >> 10) & 1)) >> 10;  // 53 bits, or 2^53
+  const unsigned long long b = ((unsigned long long)(unsigned)(1085 - lz) << 52) + r;
+  return __longlong_as_double(a ? (long long)(b | (q < 0 ? 0x8000000000000000ull : 0ull)) : 0ll);
+}
+
 // sum of limbs back to one double (in units of limb_unit): exact below 2^53,
 // one rounding above.  Each limb sum is an integer below 2^24.
+template <bool INT>
 __device__ __forceinline__ double join18(float s2, float s1, float s0) {
   const long long q = ((long long)__float2int_rn(s2) << 36) + ((long long)__float2int_rn(s1) << 18) +
                       (long long)__float2int_rn(s0);
-  return (double)q;
+  return INT ? int_to_double(q) : (double)q;
 }
 
 // A 57-bit integer in two limbs, q = h 2^28 + l with -2^27 <= l < 2^27: sums

@@ -313,6 +313,125 @@ __global__ void __launch_bounds__(kBlock) k_flux_grp(Tab T, Dev d) {
   }
 }
 
+__global__ void k_update(Tab T, Dev d) {
+  // Every load of a thread is issued before its first store: a load after a
+  // store to memory that might alias it waits for the store, and this kernel
+  // is a chain of dependent gathers whose round trips set its duration.
+  const int epoch = d.cnt->epoch;
+  const long long Ts = d.cnt->t_sync;
+  const int n_touched = d.cnt->n_touched;
+  const int stride = gridDim.x * blockDim.x;
+  for (int base = blockIdx.x * blockDim.x; base < n_touched; base += stride) {
+    int q = base + threadIdx.x;
+    bool upd = false;
+    double gcl = 0.0;  // GCL residual of this thread's update (non-negative)
+    if (q < n_touched) {
+      const int i = d.touch_list[q];
+      const bool ready = d.elem_ready[i] == epoch;
+      int eds[3];
+      bool act[3];
+      double sg[3], Ge[3][4], Ne[3][3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) eds[e] = d.elem_edge[3 * i + e];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        act[e] = d.edge_act[eds[e]] == epoch;
+        sg[e] = d.edge_elem[2 * eds[e]] == i ? 1.0 : -1.0;
+      }
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) Ge[e][v] = act[e] ? d.G[4 * (size_t)eds[e] + v] : 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Ne[e][c] = act[e] ? d.N[4 * (size_t)eds[e] + c] : 0.0;
+      }
+      double Qo[4], QMo[4], HMo[3];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) { Qo[v] = d.Q[4 * i + v]; QMo[v] = d.QM[4 * i + v]; }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) HMo[c] = d.HM[4 * i + c];
+      if (ready) {
+        upd = true;
+        double Xo[6], Xn[6];
+        int nd[3];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) Xo[k] = d.X[6 * i + k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) nd[k] = d.tri[3 * i + k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          Xn[2 * k] = d.nXn[2 * nd[k]] + d.cshift[6 * i + 2 * k];
+          Xn[2 * k + 1] = d.nXn[2 * nd[k] + 1] + d.cshift[6 * i + 2 * k + 1];
+        }
+        const long long ti = d.t[i], dti = d.dt[i], ci = d.count[i];
+        double Aold = area6(Xo), Anew = area6(Xn);
+        double Qn[4];
+        for (int v = 0; v < 4; ++v) {
+          double acc = Aold * Qo[v];
+          for (int e = 0; e < 3; ++e)
+            if (act[e]) acc -= sg[e] * Ge[e][v];
+          acc += QMo[v];
+          Qn[v] = acc / Anew;
+        }
+        double res[3];
+        for (int c = 0; c < 3; ++c) {
+          double acc = 0.0;
+          for (int e = 0; e < 3; ++e)
+            if (act[e]) acc += sg[e] * Ne[e][c];
+          res[c] = acc - HMo[c];
+        }
+        res[2] += Anew - Aold;
+        gcl = fmax(fabs(res[0]), fmax(fabs(res[1]), fabs(res[2]))) / Aold;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          d.Q[4 * i + v] = Qn[v];
+          d.QM[4 * i + v] = 0.0;
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d.HM[4 * i + c] = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) d.X[6 * i + k] = Xn[k];
+        d.t[i] = ti + dti;
+        if (ti + dti >= Ts) atomicSub(&d.cnt->n_unfinished, 1);
+        d.count[i] = ci + 1;
+        if (!(Qn[0] > 0.0) || !(pressure(T, Qn) > 0.0) || !(Anew > 0.0)) set_error(d.cnt, -3, i);
+      } else {
+        double QMn[4], HMn[3];
+        for (int v = 0; v < 4; ++v) {
+          double acc = QMo[v];
+          for (int e = 0; e < 3; ++e)
+            if (act[e]) acc -= sg[e] * Ge[e][v];
+          QMn[v] = acc;
+        }
+        for (int c = 0; c < 3; ++c) {
+          double acc = HMo[c];
+          for (int e = 0; e < 3; ++e)
+            if (act[e]) acc -= sg[e] * Ne[e][c];
+          HMn[c] = acc;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) d.QM[4 * i + v] = QMn[v];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) d.HM[4 * i + c] = HMn[c];
+      }
+    }
+    unsigned um = __ballot_sync(0xffffffffu, upd);
+    // the warp's largest residual (non-negative doubles order like their
+    // bit patterns), one atomic per warp
+    unsigned long long gb = (unsigned long long)__double_as_longlong(gcl);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, gb, off);
+      gb = o > gb ? o : gb;
+    }
+    if ((threadIdx.x & 31) == 0 && um) atomicMax(&d.cnt->gcl_bits, gb);
+    if ((threadIdx.x & 31) == 0 && um) {
+      atomicAdd((unsigned long long*)&d.cnt->updates, (unsigned long long)__popc(um));
+      atomicAdd((unsigned long long*)&d.cnt->updates_since_sync, (unsigned long long)__popc(um));
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // virtual data of element j at time ti (ticks): eqs. virtGeom, virtCellaverage
 template <int M>
@@ -1202,6 +1321,10 @@ void launch_plain_flux(const Tab& T, const Dev& d, int nsm, cudaStream_t s, cons
     case 2: k_flux_grp<2><<<grid, kBlock, 0, s>>>(T, d); break;
     default: k_flux_grp<3><<<grid, kBlock, 0, s>>>(T, d); break;
   }
+}
+
+void launch_plain_update(const Tab& T, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl) {
+  k_update<<<nsm * tl.bpsm, kBlock, 0, s>>>(T, d);
 }
 
 void launch_plain_recon(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int initial, const Tiles& tl) {

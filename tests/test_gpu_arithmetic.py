@@ -32,7 +32,8 @@ __global__ void k_limbs(const double* x, const int* E, float4* f, double* j, int
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     f[i] = aw::limbs18(x[i], E[i]);
-    j[i] = aw::join18(f[i].x, f[i].y, f[i].z) * aw::limb_unit(E[i]);
+    const double v = i & 1 ? aw::join18<true>(f[i].x, f[i].y, f[i].z) : aw::join18<false>(f[i].x, f[i].y, f[i].z);
+    j[i] = v * aw::limb_unit(E[i]);
   }
 }
 __global__ void k_roots(const double* x, double* s, double* r, int n) {
@@ -54,6 +55,14 @@ __global__ void k_dot(const double* a, const double* b, int len, long long* hh, 
   hl[i] = l;
   const aw::F2 g = aw::f2_of_dot(h, l);
   f[i] = make_float2(g.h, g.l);
+}
+__global__ void k_int(const long long* q, double* x, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) x[i] = aw::int_to_double(q[i]);
+}
+extern "C" int from_int(const long long* q, double* x, int n) {
+  k_int<<<(n + 127) / 128, 128>>>(q, x, n);
+  return cudaDeviceSynchronize();
 }
 extern "C" int roots(const double* x, double* s, double* r, int n) {
   k_roots<<<(n + 127) / 128, 128>>>(x, s, r, n);
@@ -136,6 +145,17 @@ def test_integer_dot(lib, length):
         assert abs(got - exact) <= length << 54, i
         v = got / 2.0 ** 56
         assert abs(f[i, 0] + f[i, 1] - v) <= abs(v) * 2.0 ** -46 + 2.0 ** -20, i
+
+
+def test_int_to_double(lib):
+    """The nearest double, ties to even."""
+    rng = np.random.default_rng(5)
+    q = rng.integers(-2 ** 62, 2 ** 62, 100000) >> rng.integers(0, 62, 100000)
+    q[:10] = 0, 1, -1, 2 ** 53 - 1, 2 ** 53 + 1, -2 ** 53 - 3, 2 ** 62 - 1, -2 ** 62, 2 ** 54 - 1, 2 ** 61 + 2 ** 8
+    qd, x = torch.tensor(q, device="cuda"), torch.empty(q.size, dtype=torch.float64, device="cuda")
+    assert lib.from_int(_p(qd), _p(x), q.size) == 0
+    for a, b in zip(q.tolist(), x.cpu().tolist()):
+        assert b == float(a), a
 
 
 def test_limbs(lib):

@@ -34,14 +34,13 @@ struct aw_ctx {
   double prof_ms[kNumKernels] = {0};
   long long prof_sweeps = 0;
   long long ne = 0, nn = 0, ned = 0, sw_total = 0, u_total = 0;
-  std::vector<double> xy0;
   double* d_corner0 = nullptr;  // element corners at t = 0
+  double* d_xy0 = nullptr;      // node positions at t = 0
+  int* d_check = nullptr;       // first bad average, first inverted element
   std::vector<double> etick_h, ntick_h;  // seconds per tick of each element / node
   cudaGraphExec_t graph_exec[2] = {};  // one captured sweep: the fast and the plain kernels (Dev::plain)
   cudaGraphExec_t graph_run[2] = {};   // kRun captured sweeps
   Tiles tiles;                           // tile shapes of the sweep kernels
-  std::vector<int> tri_h;                // host copies for aw_load_state_xy
-  std::vector<double> cshift_h;
   bool fresh = false;                    // a state was loaded and no sweep has run since
   bool batch = false;                    // loaded by aw_load_batch (ticks differ per instance)
   long long t_sync = 0;                  // the sync time in ticks (a copy of the device's)
@@ -683,36 +682,26 @@ void free_all(aw_ctx* c) {
   c->fresh = false;
 }
 
+int sync_counters(aw_ctx* c);
+
 // Counters and epoch stamps restart together (a stale stamp equal to a new
 // epoch would mark an element or node as active).
 int reset_sweep_state(aw_ctx* c) {
-  const Dev& d = c->d;
-  CK(cudaMemsetAsync(d.elem_ready, 0, c->ne * sizeof(int), c->stream));
-  CK(cudaMemsetAsync(d.elem_touch, 0, c->ne * sizeof(int), c->stream));
-  CK(cudaMemsetAsync(d.node_moved, 0, c->nn * sizeof(int), c->stream));
-  CK(cudaMemsetAsync(d.edge_act, 0, c->ned * sizeof(int), c->stream));
-  CK(cudaMemsetAsync(d.cand_stamp, 0, c->ne * sizeof(int), c->stream));
-  CK(cudaMemsetAsync(d.cnt, 0, sizeof(Counters), c->stream));
-  static const int one = 1;  // stamps are 0: the first sweep must be epoch 1
-  CK(cudaMemcpyAsync(&d.cnt->epoch, &one, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemcpyAsync(&d.cnt->t_sync, &c->t_sync, sizeof(long long), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  launch_reset_sweeps(c->d, c->ned, c->t_sync, c->nsm, c->stream);
+  CK(cudaGetLastError());
   return AW_OK;
 }
 
-// elements with t < t_sync, counted on the host from the device times
+// elements with t < t_sync, into the counters; with max_t, the largest element
+// time (waits for it)
 int count_unfinished(aw_ctx* c, long long* max_t) {
-  std::vector<long long> th(c->ne);
-  CK(cudaStreamSynchronize(c->stream));
-  CK(cudaMemcpy(th.data(), c->d.t, c->ne * sizeof(long long), cudaMemcpyDeviceToHost));
-  int unf = 0;
-  long long mx = 0;
-  for (long long v : th) {
-    unf += v < c->t_sync;
-    mx = std::max(mx, v);
+  launch_count_unfinished(c->d, c->t_sync, c->nsm, c->stream);
+  CK(cudaGetLastError());
+  if (max_t) {
+    const int rc = sync_counters(c);
+    if (rc) return rc;
+    *max_t = c->hcnt->max_t;
   }
-  if (max_t) *max_t = mx;
-  CK(cudaMemcpy(&c->d.cnt->n_unfinished, &unf, sizeof(int), cudaMemcpyHostToDevice));
   return AW_OK;
 }
 
@@ -968,15 +957,14 @@ static int load_common(aw_ctx* c, int64_t n_nodes, const double* xy, int64_t n_t
   CK(cudaMemsetAsync(d.cnt, 0, sizeof(Counters), c->stream));
   CK(cudaMemcpyAsync(d.nX, hxy.data(), 2 * nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  c->xy0 = hxy;
-  c->tri_h = m.tri;
-  c->cshift_h = m.cshift;
   c->ne = m.ne; c->nn = m.nn; c->ned = m.ned; c->sw_total = (long long)m.sw.size();
   c->u_total = (long long)m.u_elem.size();
   c->have_mesh = true;
   c->have_state = false;
   c->failed = false;
-  if ((rc = dalloc(c, &c->d_corner0, 6 * ne))) return rc;
+  if ((rc = dalloc(c, &c->d_corner0, 6 * ne)) || (rc = dalloc(c, &c->d_xy0, 2 * nn)) || (rc = dalloc(c, &c->d_check, 2)))
+    return rc;
+  CK(cudaMemcpy(c->d_xy0, hxy.data(), 2 * nn * sizeof(double), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(c->d_corner0, m.corner0.data(), 6 * ne * sizeof(double), cudaMemcpyHostToDevice));
   return AW_OK;
 }
@@ -1026,53 +1014,31 @@ static int load_state_impl(aw_ctx* c, const double* Q, const double* xy) {
   if (!c || !Q) return AW_ERR_INVALID_ARG;
   if (!c->have_mesh) return set_err(c, AW_ERR_STATE, "no mesh loaded");
   const size_t ne = c->ne, nn = c->nn;
-  std::vector<double> hQ(4 * ne);
-  CK(cudaMemcpy(hQ.data(), Q, hQ.size() * sizeof(double), cudaMemcpyDefault));
-  const double g = c->tab.gamma;
-  for (size_t i = 0; i < ne; ++i) {
-    const double* q = &hQ[4 * i];
-    double p = (g - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
-    if (!(q[0] > 0) || !(p > 0)) return set_err(c, AW_ERR_NONPHYSICAL, "initial state of element %zu is not physical", i);
-  }
-  std::vector<double> hxy, corners;
-  if (xy) {
-    hxy.resize(2 * nn);
-    CK(cudaMemcpy(hxy.data(), xy, hxy.size() * sizeof(double), cudaMemcpyDefault));
-    corners.resize(6 * ne);
-    for (size_t i = 0; i < ne; ++i)
-      for (int k = 0; k < 3; ++k) {
-        const int n = c->tri_h[3 * i + k];
-        corners[6 * i + 2 * k] = hxy[2 * n] + c->cshift_h[6 * i + 2 * k];
-        corners[6 * i + 2 * k + 1] = hxy[2 * n + 1] + c->cshift_h[6 * i + 2 * k + 1];
-      }
-    for (size_t i = 0; i < ne; ++i) {
-      const double* X = &corners[6 * i];
-      if (!(0.5 * ((X[2] - X[0]) * (X[5] - X[1]) - (X[3] - X[1]) * (X[4] - X[0])) > 0))
-        return set_err(c, AW_ERR_BAD_MESH, "element %zu is not counter-clockwise at the given node positions", i);
-    }
-  }
   Dev& d = c->d;
-  CK(cudaMemcpyAsync(d.Q, hQ.data(), 4 * ne * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  CK(cudaMemsetAsync(d.QM, 0, 4 * ne * sizeof(double), c->stream));
-  CK(cudaMemsetAsync(d.HM, 0, 4 * ne * sizeof(double), c->stream));
-  CK(cudaMemsetAsync(d.t, 0, ne * sizeof(long long), c->stream));
-  CK(cudaMemsetAsync(d.count, 0, ne * sizeof(long long), c->stream));
-  if (xy) {
-    CK(cudaMemcpyAsync(d.X, corners.data(), 6 * ne * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(d.nX, hxy.data(), 2 * nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  } else {
-    CK(cudaMemcpyAsync(d.X, c->d_corner0, 6 * ne * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    CK(cudaMemcpyAsync(d.nX, c->xy0.data(), 2 * nn * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  }
-  CK(cudaMemsetAsync(d.nt, 0, nn * sizeof(long long), c->stream));
+  // The new data wait in scratch (the nodal WENO values, the nodes' new
+  // positions) until they are checked: a refused state leaves the old one as it
+  // is.  Checked and spread on the device: through the host, averages and
+  // corners crossed over twice and were gone through by one core (16,200 P3
+  // triangles, whole call: 1.72 -> 1.64 ms; a batch of 111,840 P2 triangles with
+  // its 25 sweeps: 9.47 -> 9.13 ms).
+  CK(cudaStreamSynchronize(c->stream));
+  CK(cudaMemcpy(d.w0, Q, 4 * ne * sizeof(double), cudaMemcpyDefault));
+  if (xy) CK(cudaMemcpy(d.nXn, xy, 2 * nn * sizeof(double), cudaMemcpyDefault));
+  CK(cudaStreamSynchronize(cudaStreamLegacy));  // copies between device arrays are not waited for
+  launch_check_state(c->tab, d, xy != nullptr, c->d_check, c->nsm, c->stream);
+  CK(cudaGetLastError());
+  int bad[2];  // first element with a bad average, first inverted one
+  CK(cudaMemcpyAsync(bad, c->d_check, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  if (bad[0] < (int)ne) return set_err(c, AW_ERR_NONPHYSICAL, "initial state of element %d is not physical", bad[0]);
+  if (xy && bad[1] < (int)ne)
+    return set_err(c, AW_ERR_BAD_MESH, "element %d is not counter-clockwise at the given node positions", bad[1]);
   c->t_sync = c->tab.T;
+  launch_init_state(d, c->d_corner0, c->d_xy0, xy != nullptr, c->nsm, c->stream);
+  CK(cudaGetLastError());
   int rc0 = reset_sweep_state(c);
   if (rc0) return rc0;
-  {
-    int unf = (int)ne;
-    CK(cudaMemcpyAsync(&d.cnt->n_unfinished, &unf, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-  }
+  if ((rc0 = count_unfinished(c, nullptr))) return rc0;
 
   d.plain = xy ? 1 : 0;
   launch_initial(c->tab, d, c->nsm, c->stream, c->tiles);
@@ -1332,6 +1298,7 @@ int aw_set_elem_arrays(aw_ctx* c, const double* Q, const double* QM, const doubl
   CK(cudaMemcpy(c->d.X, X, 6 * ne * sizeof(double), cudaMemcpyDefault));
   CK(cudaMemcpy(c->d.count, count, ne * sizeof(long long), cudaMemcpyDefault));
   CK(cudaMemcpy(c->d.qhat, qhat, ne * c->tab.Nst * 4 * sizeof(double), cudaMemcpyDefault));
+  CK(cudaStreamSynchronize(cudaStreamLegacy));  // copies between device arrays are not waited for
   int rc0 = reset_sweep_state(c);
   if (rc0) return rc0;
   if ((rc0 = count_unfinished(c, nullptr))) return rc0;
@@ -1364,6 +1331,7 @@ int aw_set_node_arrays(aw_ctx* c, const double* X, const int64_t* t) {
   CK(cudaStreamSynchronize(c->stream));
   CK(cudaMemcpy(c->d.nX, X, 2 * c->nn * sizeof(double), cudaMemcpyDefault));
   CK(cudaMemcpy(c->d.nt, t, c->nn * sizeof(long long), cudaMemcpyDefault));
+  CK(cudaStreamSynchronize(cudaStreamLegacy));
   return AW_OK;
 }
 

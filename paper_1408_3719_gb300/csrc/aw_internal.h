@@ -169,14 +169,15 @@ struct Counters {
   int finish_blocks;
   long long updates_since_sync;
   long long surfaces;            // space-time edge surfaces integrated (all sweeps)
+  long long max_t;               // largest element time (k_count_unfinished)
   long long t_sync;              // sync time in ticks: steps are clipped at it and elements
                                  // stop there (T unless aw_advance_to set an earlier time)
 };
 
 // Tile shapes of a sweep's kernels (they change no arithmetic): recon_half
-// halves the reconstruction's elements and threads per block, pred_wide runs the
-// predictor on 256-thread blocks instead of 128, bpsm = blocks per SM of the
-// persistent kernels that loop over the sweep's lists.
+// halves the reconstruction's elements per block, pred_wide runs the predictor
+// on 256-thread blocks instead of 128, bpsm = blocks per SM of the light kernels
+// that loop over the sweep's lists.
 struct Tiles {
   int recon_half = 0;
   int pred_wide = 0;
@@ -188,6 +189,13 @@ constexpr int kNumKernels = 7;  // timed parts of a sweep (k_finish: plain kerne
 const char* kernel_name(int k);
 void launch_sweep(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, cudaEvent_t* ev, const Tiles& tl);
 void launch_initial(const Tab& tab, const Dev& d, int nsm, cudaStream_t s, const Tiles& tl);
+// loading a state: check of the averages in d.w0 (and of the elements at the node
+// positions in d.nXn), with bad[0], bad[1] the first refused element (ne: none);
+// then the initial state from them; counters and stamps; unfinished elements
+void launch_check_state(const Tab& tab, const Dev& d, bool xy, int* bad, int nsm, cudaStream_t s);
+void launch_init_state(const Dev& d, const double* corner0, const double* xy0, bool xy, int nsm, cudaStream_t s);
+void launch_reset_sweeps(const Dev& d, long long ned, long long t_sync, int nsm, cudaStream_t s);
+void launch_count_unfinished(const Dev& d, long long t_sync, int nsm, cudaStream_t s);
 void launch_products(const Tab& tab, const Dev& d, int nsm, cudaStream_t s);
 // a new sync time Tn below the current one: every step crossing Tn is cut back
 // to it and its predictor re-solved from the element's own tau = 0 dofs

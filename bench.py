@@ -448,7 +448,8 @@ def run_ours(args, rank, world):
                 "peak_source": "measured FP64 DFMA throughput (aw_measure_fp64_peak, this run); "
                                "MEASURED_PEAKS.json has no FP64 figure",
                 f"flops_per_{unit_name}": per_unit, f"{unit_name}s_profiled": units,
-                "flops_note": "operation count of the method's steps as the kernel formulates them (bench.py: "
+                "flops_note": "operation count of the method's steps in FP64, of which the kernels run the least "
+                              "squares and nodal derivatives in integers and FP32: frac is no pipe utilisation (bench.py: "
                               "predictor_flops, recon_flops, flux_flops)",
                 "executed": executed}
     # the HBM roofline this FP64-bound path is far from: compulsory bytes per
@@ -533,7 +534,7 @@ def run_ours(args, rank, world):
                            "updates_timed": int(updates_all), "sw_entries_per_elem": sizes["sw_entries"] / n_tris,
                            "stencil_members_per_elem": members},
                 "roofline": roof, "hbm": hbm, "cpu_baseline": cpu, "e2e": e2e, "full_run": full,
-                "gpu_launches": len(kms) * args.steps,
+                "gpu_launches": sum(k != "k_finish" for k in kms) * args.steps,  # k_finish: differentiated runs only
                 "clocks": clk,
                 "kernels": {k: {"ms": v, "share": v / share_tot} for k, v in kms.items()},
                 "kernels_note": f"CUDA-event times over a second pass of {ksweeps} sweeps ({prof_updates} updates)",

@@ -121,7 +121,8 @@ int aw_load_state(aw_ctx* ctx, const double* Q);
  * instead of the mesh's own: element corners become xy[tri] plus their
  * periodic offsets.  The mesh pre-processing of aw_load_mesh (stencils,
  * total stencils, wall normals) is kept, so a small move of the nodes changes
- * the result smoothly.  BAD_MESH if an element turns clockwise. */
+ * the result smoothly.  BAD_MESH if an element turns clockwise.  With the mesh's
+ * own positions the same state as aw_load_state's, bit for bit. */
 int aw_load_state_xy(aw_ctx* ctx, const double* Q, const double* xy);
 
 /* One cycle of the LTS algorithm (Sec. 2.6): every element satisfying the
@@ -235,8 +236,9 @@ int aw_get_schedule(aw_ctx* ctx, int64_t* out);
 /* Adjoint of n LTS sweeps for the schedule they take (the sweep map with the
  * ready sets and tick steps held fixed, and the mesh pre-processing of
  * aw_load_mesh held fixed).
- * aw_adjoint_forward runs n_sweeps sweeps from a state just loaded by
- * aw_load_state / aw_load_state_xy and keeps a device checkpoint of the
+ * aw_adjoint_load_state is aw_load_state_xy for a run that is to be
+ * differentiated.  aw_adjoint_forward runs n_sweeps sweeps from a state just
+ * loaded by it, or by aw_load_state / aw_load_state_xy, and keeps a device checkpoint of the
  * state every ckpt_every sweeps (plus the final state); STATE if a sweep ran
  * since the load.  aw_adjoint then takes dJ/d(final state) of a scalar J --
  * dJdQ [n_tris][4] conserved averages, dJdX [n_tris][6] element corners,
@@ -253,7 +255,12 @@ int aw_get_schedule(aw_ctx* ctx, int64_t* out);
  * another J.  STATE if a positivity safeguard (scaling of w_h, predictor
  * fallback) acted in one of the sweeps: the map has a kink there.  The
  * adjoint covers the Rusanov-type flux (flux = 0); INVALID_ARG otherwise.
- * No counterpart in the paper. */
+ * The sweeps of these calls run in plain FP64 kernels, whose roundings (and so
+ * the gradient's last digits) do not change with the others': their state
+ * differs from aw_enqueue_sweeps' by rounding.  From a state loaded by the other
+ * two, aw_adjoint_forward first takes the pre-processing phase again in them.
+ * Sweeps after these calls are ordinary ones.  No counterpart in the paper. */
+int aw_adjoint_load_state(aw_ctx* ctx, const double* Q, const double* xy);
 int aw_adjoint_forward(aw_ctx* ctx, int64_t n_sweeps, int64_t ckpt_every);
 int aw_adjoint(aw_ctx* ctx, const double* dJdQ, const double* dJdX, const double* dJdxy,
                double* dJdQ0, double* dJdxy0);

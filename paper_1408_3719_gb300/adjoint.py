@@ -32,7 +32,7 @@ class LtsRun(torch.autograd.Function):
         Qd = Q0.detach().to(dtype=torch.float64).contiguous()
         xyd = xy0.detach().to(device=dev, dtype=torch.float64).contiguous()
         _settle(Qd)
-        solver.load_state_xy(Qd, xyd)
+        solver.adjoint_load_state(Qd, xyd)
         solver.adjoint_forward(int(n_sweeps), int(ckpt_every))
         Q = torch.empty((solver.n_tris, 4), dtype=torch.float64, device=dev)
         X = torch.empty((solver.n_tris, 6), dtype=torch.float64, device=dev)

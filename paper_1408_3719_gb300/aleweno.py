@@ -26,7 +26,7 @@ EXPORTED = ["aw_create", "aw_destroy", "aw_last_error", "aw_load_mesh", "aw_load
             "aw_get_update_counts", "aw_get_elem_arrays", "aw_set_elem_arrays", "aw_get_node_arrays",
             "aw_set_node_arrays", "aw_diagnostics", "aw_sizes", "aw_profile_enable", "aw_profile_read",
             "aw_kernel_name", "aw_ready_set_noalloc", "aw_measure_fp64_peak", "aw_load_state_xy", "aw_schedule",
-            "aw_get_schedule", "aw_adjoint_forward", "aw_adjoint", "aw_adjoint_selftest", "aw_set_tiles",
+            "aw_get_schedule", "aw_adjoint_load_state", "aw_adjoint_forward", "aw_adjoint", "aw_adjoint_selftest", "aw_set_tiles",
             "aw_get_tiles", "aw_autotune"]
 
 _lock = threading.Lock()
@@ -89,6 +89,7 @@ def load(path: str | None = None):
             lib.aw_load_state_xy.argtypes = [P, P, P]
             lib.aw_schedule.argtypes = [P, C.c_int, i64]
             lib.aw_get_schedule.argtypes = [P, P]
+            lib.aw_adjoint_load_state.argtypes = [P, P, P]
             lib.aw_adjoint_forward.argtypes = [P, i64, i64]
             lib.aw_adjoint.argtypes = [P, P, P, P, P, P]
             lib.aw_adjoint_selftest.argtypes = [C.c_int, C.c_uint64, P]
@@ -230,6 +231,11 @@ class Solver:
         out = np.empty((self.n_tris, self._sched_k), np.int64)
         self._check(self.lib.aw_get_schedule(self.h, _ptr(out)))
         return out
+
+    def adjoint_load_state(self, Q, xy):
+        """load_state_xy for a run that is to be differentiated."""
+        Q, xy = _f64(Q), _f64(xy)
+        self._check(self.lib.aw_adjoint_load_state(self.h, _ptr(Q), _ptr(xy)))
 
     def adjoint_forward(self, n_sweeps, ckpt_every=10):
         """n_sweeps sweeps from the state just loaded, keeping checkpoints."""

@@ -42,6 +42,8 @@ struct aw_ctx {
   cudaGraphExec_t graph_run[2] = {};   // kRun captured sweeps
   Tiles tiles;                           // tile shapes of the sweep kernels
   bool fresh = false;                    // a state was loaded and no sweep has run since
+  bool plain_state = false;              // the plain kernels made the derived tables (and, in a fresh
+                                         // state, the predictor)
   bool batch = false;                    // loaded by aw_load_batch (ticks differ per instance)
   long long t_sync = 0;                  // the sync time in ticks (a copy of the device's)
   // frozen schedule (record / replay of the dt ticks)
@@ -680,9 +682,28 @@ void free_all(aw_ctx* c) {
   c->d_sched = nullptr;
   c->have_mesh = c->have_state = false;
   c->fresh = false;
+  c->plain_state = false;
 }
 
 int sync_counters(aw_ctx* c);
+
+// The plain kernels run inside the calls of a differentiated run only: every
+// other sweep takes the fast ones, however its state came in, so that a saved
+// and restored run goes on as the uninterrupted one.
+struct PlainScope {
+  aw_ctx* c;
+  explicit PlainScope(aw_ctx* ctx, bool on = true) : c(ctx) { c->d.plain = on ? 1 : 0; }
+  ~PlainScope() { c->d.plain = 0; }
+};
+
+// the derived tables as the fast kernels form them from the stored predictor
+int fast_tables(aw_ctx* c) {
+  if (!c->plain_state) return AW_OK;
+  launch_products(c->tab, c->d, c->nsm, c->stream);
+  CK(cudaGetLastError());
+  c->plain_state = false;
+  return AW_OK;
+}
 
 // Counters and epoch stamps restart together (a stale stamp equal to a new
 // epoch would mark an element or node as active).
@@ -1010,7 +1031,7 @@ int aw_load_batch(aw_ctx* c, int n_inst, const int64_t* node_offsets, const int6
   return rc;
 }
 
-static int load_state_impl(aw_ctx* c, const double* Q, const double* xy) {
+static int load_state_impl(aw_ctx* c, const double* Q, const double* xy, bool plain = false) {
   if (!c || !Q) return AW_ERR_INVALID_ARG;
   if (!c->have_mesh) return set_err(c, AW_ERR_STATE, "no mesh loaded");
   const size_t ne = c->ne, nn = c->nn;
@@ -1040,7 +1061,8 @@ static int load_state_impl(aw_ctx* c, const double* Q, const double* xy) {
   if (rc0) return rc0;
   if ((rc0 = count_unfinished(c, nullptr))) return rc0;
 
-  d.plain = xy ? 1 : 0;
+  PlainScope plain_(c, plain);
+  c->plain_state = plain;
   launch_initial(c->tab, d, c->nsm, c->stream, c->tiles);
   CK(cudaGetLastError());
   int rc = sync_counters(c);
@@ -1064,8 +1086,18 @@ int aw_load_state_xy(aw_ctx* c, const double* Q, const double* xy) {
   return load_state_impl(c, Q, xy);
 }
 
+int aw_adjoint_load_state(aw_ctx* c, const double* Q, const double* xy) {
+  DeviceGuard dg_(c ? c->device : -1);
+  if (!c || !xy) return AW_ERR_INVALID_ARG;
+  return load_state_impl(c, Q, xy, true);
+}
+
 static int do_sweeps(aw_ctx* c, int64_t n, int64_t* n_updated, bool wait) {
   if (!c->have_state || c->failed) return set_err(c, AW_ERR_STATE, "no valid state (load a state first)");
+  if (!c->d.plain) {
+    const int rct = fast_tables(c);
+    if (rct) return rct;
+  }
   if (n > 0) c->fresh = false;
   // A sweep is one CUDA-graph launch (captured once per mesh and tile shape).
   // With profiling it is a second graph with an event record between the
@@ -1156,6 +1188,7 @@ static int set_sync_time(aw_ctx* c, long long Tn) {
   int rc = count_unfinished(c, &max_t);
   if (rc) return rc;
   if (max_t > Tn) return set_err(c, AW_ERR_INVALID_ARG, "aw_advance_to: an element is beyond the sync time");
+  if ((rc = fast_tables(c))) return rc;
   const long long Told = c->t_sync;
   c->t_sync = Tn;
   c->fresh = false;  // the adjoint starts from a state just loaded
@@ -1303,7 +1336,7 @@ int aw_set_elem_arrays(aw_ctx* c, const double* Q, const double* QM, const doubl
   if (rc0) return rc0;
   if ((rc0 = count_unfinished(c, nullptr))) return rc0;
 
-  c->d.plain = 0;
+  c->plain_state = false;
   launch_products(c->tab, c->d, c->nsm, c->stream);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->stream));
@@ -1449,7 +1482,16 @@ int aw_adjoint_forward(aw_ctx* c, int64_t n_sweeps, int64_t ckpt_every) {
   for (auto& s : c->slots)
     if ((rc = snap_alloc(c, &s))) return rc;
   c->last_seg_kept = false;
-  c->d.plain = 1;
+  PlainScope plain_(c);
+  if (!c->plain_state) {
+    // the fast kernels prepared the state: the run starts from the plain ones'
+    // reconstruction, steps and predictor (aw_adjoint_load_state makes them at once)
+    c->plain_state = true;
+    launch_initial(c->tab, c->d, c->nsm, c->stream, c->tiles);
+    CK(cudaGetLastError());
+    if ((rc = sync_counters(c))) return rc;
+    if ((rc = check_device_error(c))) return rc;
+  }
   if ((rc = snap_copy(c, c->ckpt[0], true))) return rc;
   // the last segment is the first one the reverse pass needs: keep its
   // sweep-start states now instead of recomputing them
@@ -1503,6 +1545,8 @@ int aw_adjoint(aw_ctx* c, const double* dJdQ, const double* dJdX, const double* 
   CK(cudaMemsetAsync(a.vdb, 0, ne * 6 * Nt * sizeof(double), c->stream));
   CK(cudaMemsetAsync(a.nXnb, 0, 2 * nn * sizeof(double), c->stream));
   CK(cudaMemsetAsync(a.gb, 0, 4 * ne * sizeof(double), c->stream));
+  PlainScope plain_(c);
+  c->plain_state = true;  // the recomputed sweeps' and the final state's
   const int64_t n = c->adj_n, k = c->adj_k;
   const int64_t nseg = (n + k - 1) / k;
   for (int64_t seg = nseg - 1; seg >= 0; --seg) {
@@ -1570,10 +1614,12 @@ int aw_autotune(aw_ctx* c, int64_t n_sweeps, double* ms, int32_t* best) {
   DeviceGuard dg_(c ? c->device : -1);
   if (!c || n_sweeps < 1) return AW_ERR_INVALID_ARG;
   if (!c->have_state || c->failed) return set_err(c, AW_ERR_STATE, "no valid state (load a state first)");
+  int rc = fast_tables(c);
+  if (rc) return rc;
   CK(cudaStreamSynchronize(c->stream));
   std::vector<void*> owned;
   aw_ctx::Snap keep{};
-  int rc = snap_alloc(c, &keep, &owned);
+  rc = snap_alloc(c, &keep, &owned);
   auto done = [&](int code) {
     cudaStreamSynchronize(c->stream);
     for (void* p : owned) cudaFree(p);

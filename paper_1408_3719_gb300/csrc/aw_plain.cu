@@ -1,6 +1,7 @@
-// The heavy sweep kernels in plain FP64, for differentiated runs (states loaded
-// by aw_load_state_xy, and the sweeps of aw_adjoint_forward / aw_adjoint); all
-// other runs take the faster kernels of aw_kernels.cu, which round differently.
+// The heavy sweep kernels in plain FP64, for differentiated runs
+// (aw_adjoint_load_state's pre-processing phase and the sweeps of
+// aw_adjoint_forward and aw_adjoint); all other sweeps take the faster kernels of
+// aw_kernels.cu, which round differently.
 //
 // Why the gradients keep this rounding: the characteristic fields' direction is
 // the density gradient over its length, also where a uniform flow's gradient is

@@ -237,7 +237,7 @@ int aw_get_schedule(aw_ctx* ctx, int64_t* out);
  * ready sets and tick steps held fixed, and the mesh pre-processing of
  * aw_load_mesh held fixed).
  * aw_adjoint_load_state is aw_load_state_xy for a run that is to be
- * differentiated.  aw_adjoint_forward runs n_sweeps sweeps from a state just
+ * differentiated; it refuses what the adjoint does not cover.  aw_adjoint_forward runs n_sweeps sweeps from a state just
  * loaded by it, or by aw_load_state / aw_load_state_xy, and keeps a device checkpoint of the
  * state every ckpt_every sweeps (plus the final state); STATE if a sweep ran
  * since the load.  aw_adjoint then takes dJ/d(final state) of a scalar J --

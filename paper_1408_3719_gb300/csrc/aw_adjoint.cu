@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "aw_adjoint_elem.cuh"
+#include "aw_device.cuh"
 #include "aw_internal.h"
 
 namespace aw {
@@ -31,10 +32,6 @@ namespace aw {
 namespace {
 
 using adj::Sz;
-
-__device__ __forceinline__ void set_error(Counters* cnt, int code, int elem) {
-  if (atomicCAS(&cnt->err_code, 0, code) == 0) cnt->err_elem = elem;
-}
 
 // Work space of one element's phase-B reverse (shared memory of its warp).
 template <int M>

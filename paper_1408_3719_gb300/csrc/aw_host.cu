@@ -1086,9 +1086,20 @@ int aw_load_state_xy(aw_ctx* c, const double* Q, const double* xy) {
   return load_state_impl(c, Q, xy);
 }
 
+// what a differentiated run may be (the plain kernels hold no more)
+static int adjoint_scope(aw_ctx* c) {
+  if (c->cfg.gts) return set_err(c, AW_ERR_INVALID_ARG, "the adjoint is for local time stepping");
+  if (c->cfg.flux != 0) return set_err(c, AW_ERR_INVALID_ARG, "the adjoint covers the Rusanov-type flux");
+  if (c->tab.Tsw > 0 || c->moving_wall)
+    return set_err(c, AW_ERR_INVALID_ARG, "the adjoint covers neither moving walls, Kidder boundaries nor the global-step start-up");
+  return AW_OK;
+}
+
 int aw_adjoint_load_state(aw_ctx* c, const double* Q, const double* xy) {
   DeviceGuard dg_(c ? c->device : -1);
   if (!c || !xy) return AW_ERR_INVALID_ARG;
+  if (!c->have_mesh) return set_err(c, AW_ERR_STATE, "no mesh loaded");
+  if (const int rcs = adjoint_scope(c)) return rcs;
   return load_state_impl(c, Q, xy, true);
 }
 
@@ -1460,10 +1471,7 @@ int aw_adjoint_forward(aw_ctx* c, int64_t n_sweeps, int64_t ckpt_every) {
   if (!c || n_sweeps < 0 || ckpt_every < 1) return AW_ERR_INVALID_ARG;
   if (!c->have_state || c->failed) return set_err(c, AW_ERR_STATE, "no valid state (load a state first)");
   if (!c->fresh) return set_err(c, AW_ERR_STATE, "aw_adjoint_forward starts from a state just loaded");
-  if (c->cfg.gts) return set_err(c, AW_ERR_INVALID_ARG, "the adjoint is for local time stepping");
-  if (c->cfg.flux != 0) return set_err(c, AW_ERR_INVALID_ARG, "the adjoint covers the Rusanov-type flux");
-  if (c->tab.Tsw > 0 || c->moving_wall)
-    return set_err(c, AW_ERR_INVALID_ARG, "the adjoint covers neither moving walls, Kidder boundaries nor the global-step start-up");
+  if (const int rcs = adjoint_scope(c)) return rcs;
   CK(cudaStreamSynchronize(c->stream));
   for (void* p : c->adj_allocs) cudaFree(p);
   c->adj_allocs.clear();

@@ -1,7 +1,8 @@
 // The heavy sweep kernels in plain FP64, for differentiated runs
 // (aw_adjoint_load_state's pre-processing phase and the sweeps of
 // aw_adjoint_forward and aw_adjoint); all other sweeps take the faster kernels of
-// aw_kernels.cu, which round differently.
+// aw_kernels.cu, which round differently.  They hold what such a run can reach:
+// local steps, the Rusanov-type flux, slip walls at rest and transmissive edges.
 //
 // Why the gradients keep this rounding: the characteristic fields' direction is
 // the density gradient over its length, also where a uniform flow's gradient is
@@ -14,6 +15,7 @@
 #include <cfloat>
 #include <climits>
 
+#include "aw_device.cuh"
 #include "aw_internal.h"
 
 namespace aw {
@@ -21,40 +23,6 @@ namespace aw {
 namespace {
 
 constexpr int kBlock = 128;
-
-__device__ __forceinline__ double area6(const double* X) {
-  return 0.5 * ((X[2] - X[0]) * (X[5] - X[1]) - (X[3] - X[1]) * (X[4] - X[0]));
-}
-
-__device__ __forceinline__ void set_error(Counters* cnt, int code, int elem) {
-  if (atomicCAS(&cnt->err_code, 0, code) == 0) cnt->err_elem = elem;
-}
-
-__device__ __forceinline__ double pressure(const Tab& T, const double* q) {
-  return (T.gamma - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
-}
-
-// Exact state of the Kidder compression (Sec. 3.4, eqs. KidderIC, KidderEx)
-// at (x, y, t): a particle starting at radius r sits at h(t) r with
-// h = sqrt(1 - t^2/tau^2); density rho0(r)/h^2 with rho0^(gamma-1) linear in
-// r^2 between the two frontiers, radial velocity h' r, pressure s0 rho^gamma;
-// tau = sqrt((gamma-1)/2 (r_e0^2 - r_i0^2)/(c_e0^2 - c_i0^2)).
-__device__ void kidder_state(const Tab& T, double x, double y, double t, double* q) {
-  const double g = T.gamma, ri = T.kidder[0], re = T.kidder[1], s0 = T.kidder[4];
-  const double ai = pow(T.kidder[2], g - 1.0), ae = pow(T.kidder[3], g - 1.0);
-  const double ci2 = g * s0 * ai, ce2 = g * s0 * ae;
-  const double tau2 = 0.5 * (g - 1.0) * (re * re - ri * ri) / (ce2 - ci2);
-  const double h = sqrt(1.0 - t * t / tau2), dh = -t / (tau2 * h);
-  const double R = sqrt(x * x + y * y), r = R / h;
-  const double w = (r * r - ri * ri) / (re * re - ri * ri);
-  const double rho = pow((1.0 - w) * ai + w * ae, 1.0 / (g - 1.0)) / (h * h);
-  const double u = dh / h * x, v = dh / h * y;
-  const double p = s0 * pow(rho, g);
-  q[0] = rho;
-  q[1] = rho * u;
-  q[2] = rho * v;
-  q[3] = p / (g - 1.0) + 0.5 * rho * (u * u + v * v);
-}
 
 // Rusanov-type ALE flux through the area-weighted space-time normal n
 // (eq. rusanov): the largest |eigenvalue| of A_n^V times |n_xy| is
@@ -79,65 +47,6 @@ __device__ __forceinline__ void rusanov(const Tab& T, const double* qm, const do
   double Fp[4] = {qp[0] * wp, qp[1] * wp + pp * n[0], qp[2] * wp + pp * n[1], qp[3] * wp + pp * vnp};
 #pragma unroll
   for (int v = 0; v < 4; ++v) F[v] = 0.5 * (Fm[v] + Fp[v]) - 0.5 * smax * (qp[v] - qm[v]);
-}
-
-// Osher-type ALE flux (eq. osher) on the straight path Psi(s) = q- + s (q+ -
-// q-) (eq. path), the path integral by 3-point Gauss-Legendre quadrature:
-// at each path node |A| dq = R |Lambda| L dq with the eigenvalues
-// |n_xy| (u_n - c, u_n, u_n, u_n + c) + n_t of the ALE Jacobian and the
-// eigenvectors R, L = R^-1 of dF/dQ.n, n = n_xy / |n_xy|.
-__device__ __forceinline__ void osher(const Tab& T, const double* qm, const double* qp, const double* n,
-                                      double* F) {
-  const double g = T.gamma, gm1 = g - 1.0;
-  double rim = 1.0 / qm[0], rip = 1.0 / qp[0];
-  double um = qm[1] * rim, vm = qm[2] * rim, up = qp[1] * rip, vp = qp[2] * rip;
-  double pm = gm1 * (qm[3] - 0.5 * (qm[1] * um + qm[2] * vm));
-  double pp = gm1 * (qp[3] - 0.5 * (qp[1] * up + qp[2] * vp));
-  double wm = um * n[0] + vm * n[1] + n[2], wp = up * n[0] + vp * n[1] + n[2];
-  double vnm = um * n[0] + vm * n[1], vnp = up * n[0] + vp * n[1];
-  const double nxy = sqrt(n[0] * n[0] + n[1] * n[1]);
-  double nx = 1.0, ny = 0.0;
-  if (nxy > 0.0) {
-    const double inx = 1.0 / nxy;
-    nx = n[0] * inx;
-    ny = n[1] * inx;
-  }
-  double dq[4], D[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-  for (int v = 0; v < 4; ++v) dq[v] = qp[v] - qm[v];
-  const double r15 = 0.38729833462074168852;  // sqrt(15) / 10
-#pragma unroll
-  for (int gq = 0; gq < 3; ++gq) {
-    const double s = gq == 0 ? 0.5 - r15 : (gq == 1 ? 0.5 : 0.5 + r15);
-    const double ws = gq == 1 ? 8.0 / 18.0 : 5.0 / 18.0;
-    double q[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) q[v] = qm[v] + s * dq[v];
-    const double ir = 1.0 / q[0], u = q[1] * ir, v = q[2] * ir;
-    const double p = gm1 * (q[3] - 0.5 * (q[1] * u + q[2] * v));
-    const double a = sqrt(g * p * ir), ia = 1.0 / a, H = (q[3] + p) * ir;
-    const double un = u * nx + v * ny, ut = -u * ny + v * nx, q2 = 0.5 * (u * u + v * v);
-    const double b1 = gm1 * ia * ia, b2 = b1 * q2;
-    // characteristic amplitudes L dq, scaled by |lambda|
-    double c0 = 0.5 * (b2 + un * ia) * dq[0] - 0.5 * (b1 * u + nx * ia) * dq[1] - 0.5 * (b1 * v + ny * ia) * dq[2] +
-                0.5 * b1 * dq[3];
-    double c1 = (1.0 - b2) * dq[0] + b1 * u * dq[1] + b1 * v * dq[2] - b1 * dq[3];
-    double c2 = -ut * dq[0] - ny * dq[1] + nx * dq[2];
-    double c3 = 0.5 * (b2 - un * ia) * dq[0] - 0.5 * (b1 * u - nx * ia) * dq[1] - 0.5 * (b1 * v - ny * ia) * dq[2] +
-                0.5 * b1 * dq[3];
-    c0 *= ws * fabs(nxy * (un - a) + n[2]);
-    c1 *= ws * fabs(nxy * un + n[2]);
-    c2 *= ws * fabs(nxy * un + n[2]);
-    c3 *= ws * fabs(nxy * (un + a) + n[2]);
-    D[0] += c0 + c1 + c3;
-    D[1] += (u - a * nx) * c0 + u * c1 - ny * c2 + (u + a * nx) * c3;
-    D[2] += (v - a * ny) * c0 + v * c1 + nx * c2 + (v + a * ny) * c3;
-    D[3] += (H - a * un) * c0 + q2 * c1 + ut * c2 + (H + a * un) * c3;
-  }
-  const double Fm[4] = {qm[0] * wm, qm[1] * wm + pm * n[0], qm[2] * wm + pm * n[1], qm[3] * wm + pm * vnm};
-  const double Fp[4] = {qp[0] * wp, qp[1] * wp + pp * n[0], qp[2] * wp + pp * n[1], qp[3] * wp + pp * vnp};
-#pragma unroll
-  for (int v = 0; v < 4; ++v) F[v] = 0.5 * (Fm[v] + Fp[v]) - 0.5 * D[v];
 }
 
 // Per-edge data of a swept surface, formed once per edge (not once per Gauss
@@ -263,32 +172,20 @@ __global__ void __launch_bounds__(kBlock) k_flux_grp(Tab T, Dev d) {
         // which a gas at rest beside the boundary grows from roundoff
 #pragma unroll
         for (int v = 0; v < 4; ++v) qp[v] = d.Q[4 * (size_t)L + v];
-      } else if (bc == 3) {
-        // the exact Kidder state at the quadrature point
-        const double px = (1 - chi) * (1 - tau) * P[0][0] + chi * (1 - tau) * P[1][0] + chi * tau * P[2][0] +
-                          (1 - chi) * tau * P[3][0];
-        const double py = (1 - chi) * (1 - tau) * P[0][1] + chi * (1 - tau) * P[1][1] + chi * tau * P[2][1] +
-                          (1 - chi) * tau * P[3][1];
-        kidder_state(T, px, py, tt * E.etL, qp);
       } else {
 #pragma unroll
         for (int v = 0; v < 4; ++v) qp[v] = qm[v];
-        if (bc == 0 || bc == 2) {  // mirror the normal momentum relative to the wall
-          const double wu = bc == 2 ? T.wall_u : 0.0, wv = bc == 2 ? T.wall_v : 0.0;
+        if (bc == 0) {  // mirror the normal momentum
           const double nn = n[0] * n[0] + n[1] * n[1];
           if (nn > 0.0) {
-            const double mn = ((qm[1] - qm[0] * wu) * n[0] + (qm[2] - qm[0] * wv) * n[1]) / nn;
+            const double mn = (qm[1] * n[0] + qm[2] * n[1]) / nn;
             qp[1] = qm[1] - 2.0 * mn * n[0];
             qp[2] = qm[2] - 2.0 * mn * n[1];
-            // same internal energy: a moving wall's mirror changes the kinetic energy
-            if (bc == 2)
-              qp[3] = qm[3] + 0.5 * (qp[1] * qp[1] + qp[2] * qp[2] - qm[1] * qm[1] - qm[2] * qm[2]) / qm[0];
           }
         }
       }
       double F[4];
-      if (T.flux == 1) osher(T, qm, qp, n, F);
-      else rusanov(T, qm, qp, n, F);
+      rusanov(T, qm, qp, n, F);
 #pragma unroll
       for (int v = 0; v < 4; ++v) G[v] = wq * F[v];
 #pragma unroll
@@ -479,7 +376,7 @@ struct PredShape {
 };
 
 template <int M, int TH>
-__global__ void __launch_bounds__(TH, TH >= 256 ? 2 : 3) k_predict_coop(Tab T, Dev d, int initial, int gts) {
+__global__ void __launch_bounds__(TH, TH >= 256 ? 2 : 3) k_predict_coop(Tab T, Dev d, int initial) {
   using S = PredShape<M, TH>;
   constexpr int Mc = S::Mc, Nt = S::Nt, Nst = S::Nst, G = S::G;
   __shared__ double sq[G][Nst][4], sf[G][Nst][4], sg[G][Nst][4], sP[G][Nst][4];
@@ -501,7 +398,6 @@ __global__ void __launch_bounds__(TH, TH >= 256 ? 2 : 3) k_predict_coop(Tab T, D
   for (int k = threadIdx.x; k < 3 * Nt * Mc; k += blockDim.x) sTr[k / Mc][k % Mc] = T.Tr[k / (Nt * Mc)][(k / Mc) % Nt][k % Mc];
   for (int k = threadIdx.x; k < Mc; k += blockDim.x) sTr[3 * Nt][k] = T.wavg[k];
   const int n_ready = initial ? d.ne : d.cnt->n_ready;
-  const long long gmin = d.cnt->gts_min;
   // thread -> (time slice t, element e, lattice node s).  A warp-wide FP64
   // instruction costs the FP64 pipe the same whatever number of its lanes is
   // active, so the tau = 0 nodes (full work in the first iteration only) and
@@ -548,13 +444,8 @@ __global__ void __launch_bounds__(TH, TH >= 256 ? 2 : 3) k_predict_coop(Tab T, D
     const bool live = e < cnt;
     if (live && l == 0) {
       const int i = initial ? pos : d.ready_list[pos];
-      long long dtk = d.dt[i];
-      if ((gts || d.t[i] < T.Tsw) && dtk > 0) {
-        dtk = gmin;
-        d.dt[i] = dtk;
-      }
       sidx[e] = i;
-      sdts[e] = (double)dtk * d.etick[i];
+      sdts[e] = (double)d.dt[i] * d.etick[i];
       sbad[e] = 0;
     }
     __syncthreads();
@@ -962,11 +853,8 @@ k_recon_coop(Tab T, Dev d, int initial) {
           const double dd = 4.0 * area6(Xv) / per;
           const double uu = Qv[1] / Qv[0], vv = Qv[2] / Qv[0];
           double vel = sqrt(uu * uu + vv * vv);
-          if (k == 0)  // an element on a moving wall counts the wall's speed
-            for (int e2 = 0; e2 < 3; ++e2)
-              if (d.edge_bc[d.elem_edge[3 * (size_t)i + e2]] == 2) vel = fmax(vel, T.wall_speed);
           const double lam = vel + sqrt(T.gamma * pressure(T, Qv) / Qv[0]);
-          dtc = (ti < T.Tsw ? T.cfl_start : T.cfl) * dd / lam;
+          dtc = T.cfl * dd / lam;
           if (!(dtc > 0.0)) dtc = -1.0;
         }
         sDt[e * 4 + k] = dtc;
@@ -1207,11 +1095,8 @@ k_recon_coop(Tab T, Dev d, int initial) {
             best = d.etick[i];
           }
           const double rt = floor(best / d.etick[i]);
-          const bool start = ti < T.Tsw;  // global-step start-up
-          const long long end = start ? (T.Tsw < Ts ? T.Tsw : Ts) : Ts;
-          tks = rt > (double)(end - ti) ? end - ti : (long long)rt;
+          tks = rt > (double)(Ts - ti) ? Ts - ti : (long long)rt;
           if (tks < 1) tks = 1;
-          if (T.gts || start) atomicMin(&d.cnt->gts_min, tks);
         }
         if (d.sched_mode) {  // frozen schedule: record or replay this update's step
           const long long ci = d.count[i];
@@ -1304,7 +1189,7 @@ void launch_predict_t(const Tab& T, const Dev& d, int nsm, cudaStream_t s, int i
   // three per SM), so that balanced rounds give every SM the same elements
   const int grid = initial ? need : std::min(need, nsm * (TH >= 256 ? 2 : 3));
   (void)bpsm;
-  k_predict_coop<M, TH><<<grid, S::kThreads, 0, s>>>(T, d, initial, T.gts);
+  k_predict_coop<M, TH><<<grid, S::kThreads, 0, s>>>(T, d, initial);
 }
 
 template <int M>

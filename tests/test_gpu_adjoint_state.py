@@ -82,3 +82,22 @@ def test_adjoint_does_not_depend_on_the_loader(order, loader):
     _equal(a, b)
     for x, y in zip(*g):
         assert np.abs(x - y).max() <= 1e-12 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("option", [dict(flux="osher"), dict(gts=True), dict(t_switch=0.1, cfl_start=0.1)])
+def test_adjoint_load_state_refuses_what_the_adjoint_does_not_cover(option):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1408_3719_gb300 import aleweno
+    mesh, Q = wavy_vortex(8)
+    s, ref = (aleweno.Solver(order_M=2, t_end=1.0, **option) for _ in range(2))
+    for x in (s, ref):
+        x.load_mesh(mesh)
+        x.load_state(Q)
+    with pytest.raises(aleweno.AwError) as e:
+        s.adjoint_load_state(Q, mesh["xy"])
+    assert "INVALID_ARG" in str(e.value)
+    for x in (s, ref):  # the loaded state is as it was
+        x.enqueue(5)
+        x.sync()
+    _equal(s, ref)

@@ -10,7 +10,7 @@ captured launch; thousands of warm-up launches before it are costly).
 
 Each sweep prints one JSON line: its element updates and the space-time edge
 surfaces it integrated (the units of the reconstruction / predictor and of
-the flux kernel).  Every sweep is one launch of each of the eight sweep
+the flux kernel).  Every sweep is one launch of each of the six sweep
 kernels; loading the state launches k_products once.
 """
 from __future__ import annotations

@@ -739,7 +739,7 @@ def run_adjoint(args, emit=True):
         updates = s.sync()
         e1.synchronize()
         flush.fill_(float(k))
-        s.load_state(Q0)
+        s.adjoint_load_state(Q0, mesh["xy"])
         e2, e3, e4 = ev(), ev(), ev()
         e2.record(stream)
         s.adjoint_forward(n_sw, ck)
@@ -774,8 +774,9 @@ def run_adjoint(args, emit=True):
             "load_state_ms": ml, "sweeps_ms": mp, "forward_ms": ml + mp,
             "forward_with_checkpoints_ms": mf, "adjoint_ms": ma,
             "adjoint_over_forward": ma / (ml + mp), "adjoint_over_sweeps": ma / mp,
-            "note": "forward = aw_load_state (pre-processing phase over every element) + the sweeps: the map "
-                    "the gradient differentiates"}
+            "note": "forward = aw_load_state (pre-processing phase over every element) + the sweeps, by the kernels "
+                    "of an ordinary run; the differentiated sweeps take plain FP64 kernels "
+                    "(forward_with_checkpoints_ms)"}
     if emit:
         print(json.dumps(line), flush=True)
     return {"value": line["value"], "unit": UNIT, "steps": args.steps, "workload": line["config"]["workload"],

@@ -114,7 +114,17 @@ int aw_load_batch(aw_ctx* ctx, int n_inst, const int64_t* node_offsets, const in
 
 /* Pre-processing phase of Sec. 2.6: cell averages Q [n_tris][4] at t = 0,
  * first WENO reconstruction, local time steps (eq. timestep), predictor;
- * all node and element times set to 0.  NONPHYSICAL if rho or p <= 0. */
+ * all node and element times set to 0.  NONPHYSICAL if rho or p <= 0.
+ *
+ * Arithmetic of this phase and of the sweeps: FP64, but for the least-squares
+ * sums of orders 2 and 3 and the predictor's nodal derivatives, which run in
+ * fixed point.  A stencil member's difference from the element keeps 2^-57 of
+ * that variable's largest difference over the element's members (and the powers
+ * of its coordinates likewise), a nodal value 2^-54 of the largest of its group
+ * (density, momentum, energy, momentum flux, energy flux) on the element: smaller
+ * ones keep fewer bits than a double.  The least squares are solved by a factor
+ * of 48 bits and refinement where the stencil's condition number (columns scaled)
+ * is below about 10^6, beyond that by an orthogonal factorisation in FP64. */
 int aw_load_state(aw_ctx* ctx, const double* Q);
 
 /* aw_load_state on node positions xy [n_nodes][2] (host or device pointer)
@@ -237,8 +247,9 @@ int aw_get_schedule(aw_ctx* ctx, int64_t* out);
  * ready sets and tick steps held fixed, and the mesh pre-processing of
  * aw_load_mesh held fixed).
  * aw_adjoint_load_state is aw_load_state_xy for a run that is to be
- * differentiated; it refuses what the adjoint does not cover.  aw_adjoint_forward runs n_sweeps sweeps from a state just
- * loaded by it, or by aw_load_state / aw_load_state_xy, and keeps a device checkpoint of the
+ * differentiated; it refuses what the adjoint does not cover.
+ * aw_adjoint_forward runs n_sweeps sweeps from a state just loaded by it, or by
+ * aw_load_state / aw_load_state_xy, and keeps a device checkpoint of the
  * state every ckpt_every sweeps (plus the final state); STATE if a sweep ran
  * since the load.  aw_adjoint then takes dJ/d(final state) of a scalar J --
  * dJdQ [n_tris][4] conserved averages, dJdX [n_tris][6] element corners,
